@@ -28,15 +28,26 @@ __device__ __forceinline__ float sigmoid_rate(float u, float beta, float theta) 
     return 1.0f / (1.0f + expf(-beta * (u - theta)));
 }
 
-// vg[b, i] = (dt b4 lam_i, q_i f(U_i))  -- entering the last stage of a step
+// The adjoint state (lam, acc, nu, the stage inputs) lives in the operator's node order; only
+// lambda_T, the checkpoints and grad_u0 are in the caller's.
+__global__ void adj_gather_kernel(const float *__restrict__ src, const int *__restrict__ perm, int64_t n, int B,
+                                  float *__restrict__ dst) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (int64_t)B * n) return;
+    const int64_t b = idx / n;
+    dst[idx] = src[b * n + perm[idx - b * n]];
+}
+
+// nu[b, i] = dt b4 lam_i, g[b, i] = q_i f(U_i)  -- entering the last stage of a step
 __global__ void adj_prep_kernel(const float *__restrict__ lam, const float *__restrict__ U, const float *__restrict__ q,
                                 const float *__restrict__ beta, const float *__restrict__ theta, int64_t n,
-                                int64_t n_pad, int B, float dtb4, float2 *__restrict__ vg) {
+                                int64_t n_pad, int B, float dtb4, float *__restrict__ nu, float *__restrict__ g) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)B * n) return;
     const int b = (int)(idx / n);
     const int64_t i = idx - (int64_t)b * n;
-    vg[(int64_t)b * n_pad + i] = make_float2(dtb4 * lam[idx], q[i] * sigmoid_rate(U[idx], beta[b], theta[b]));
+    nu[(int64_t)b * n_pad + i] = dtb4 * lam[idx];
+    g[(int64_t)b * n_pad + i] = q[i] * sigmoid_rate(U[idx], beta[b], theta[b]);
 }
 
 struct AdjEpiArgs {
@@ -48,8 +59,10 @@ struct AdjEpiArgs {
     const float *Ucur;       // U_s
     const float *Uprev;      // U_{s-1} (stg > 0), U_4 of the previous step (stg == 0), or null
     float *lam, *acc;
-    float2 *vg;
+    float *nu, *g;           // B x n_pad each
     const float *q, *beta, *theta;
+    const int *perm;         // caller's node of each position
+    float *out;              // dL/du_0 in the caller's order (the last stage of all), or null
     float dt;
 };
 
@@ -60,7 +73,7 @@ __global__ void adj_epilogue_kernel(AdjEpiArgs a) {
     const int64_t i = idx - (int64_t)b * a.n;
     const float Wnu = sum_slots(a.wpart + (int64_t)b * a.n_pad + i, (int64_t)a.B * a.n_pad, a.slots);
     const int64_t vi = (int64_t)b * a.n_pad + i;
-    const float nu = a.vg[vi].x;
+    const float nu = a.nu[vi];
     const float bb = a.beta[b], th = a.theta[b];
     const float f = sigmoid_rate(a.Ucur[idx], bb, th);
     const float fp = a.q[i] * bb * f * (1.f - f);
@@ -71,12 +84,16 @@ __global__ void adj_epilogue_kernel(AdjEpiArgs a) {
         const float accv = (a.stg == 3) ? mu : a.acc[idx] + mu;
         a.acc[idx] = accv;
         const float nun = a.dt * bw[a.stg - 1] * a.lam[idx] + cprev[a.stg] * a.dt * mu;
-        a.vg[vi] = make_float2(nun, a.q[i] * sigmoid_rate(a.Uprev[idx], bb, th));
+        a.nu[vi] = nun;
+        a.g[vi] = a.q[i] * sigmoid_rate(a.Uprev[idx], bb, th);
     } else {
         const float lamn = a.lam[idx] + (a.acc[idx] + mu);
         a.lam[idx] = lamn;
-        if (a.Uprev)
-            a.vg[vi] = make_float2(a.dt * bw[3] * lamn, a.q[i] * sigmoid_rate(a.Uprev[idx], bb, th));
+        if (a.out) a.out[(int64_t)b * a.n + a.perm[i]] = lamn;
+        if (a.Uprev) {
+            a.nu[vi] = a.dt * bw[3] * lamn;
+            a.g[vi] = a.q[i] * sigmoid_rate(a.Uprev[idx], bb, th);
+        }
     }
 }
 
@@ -189,7 +206,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
     const bool cull = op->mf_cull && op->adj_pairs;
     const int Cseg = std::min(C, std::max(nsteps, 1));
     float *stages = nullptr, *lam = nullptr, *acc = nullptr, *ubuf = nullptr, *wpart = nullptr, *gpart = nullptr;
-    float2 *vg = nullptr;
+    float *nu = nullptr;
     double *gk = nullptr;
     StreamScratch scratch(s);  // freed (stream-ordered) on every return below
     // two stage buffers: segment k - 1 is recomputed into one while segment k is reversed
@@ -202,20 +219,23 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
     // W nu slots and parameter partials for the smallest node block the kernel may take
     NF_CUDA_TRY(scratch.alloc(&wpart, sizeof(float) * (size_t)adj_slot_capacity(op) * B * n_pad));
     NF_CUDA_TRY(scratch.alloc(&gpart, sizeof(float) * 4 * (size_t)B * adj_pair_capacity(op)));
-    NF_CUDA_TRY(scratch.alloc(&vg, sizeof(float2) * (size_t)B * n_pad));
+    const size_t BP = (size_t)B * n_pad;
+    NF_CUDA_TRY(scratch.alloc(&nu, sizeof(float) * 2 * BP));
+    float *const gv = nu + BP;
     NF_CUDA_TRY(scratch.alloc(&gk, sizeof(double) * 4 * B));
-    NF_CUDA_TRY(cudaMemsetAsync(vg, 0, sizeof(float2) * (size_t)B * n_pad, s));  // padded columns stay zero
-    NF_TRY(adj_autotune(op, vg, B, wpart, gpart, s));  // first call on this operator only
+    NF_CUDA_TRY(cudaMemsetAsync(nu, 0, sizeof(float) * 2 * BP, s));  // padded columns stay zero
+    NF_TRY(adj_autotune(op, nu, gv, B, wpart, gpart, s));  // first call on this operator only
     const int slots = adj_slots(op);  // one W nu slot per node block of the chosen shape
-    const int64_t ncta = sym_pair_count(op);
+    const int64_t ncta = adj_pair_count(op);
     const int64_t ncta_run = cull ? op->adj_live : ncta;
     NF_CUDA_TRY(cudaMemsetAsync(gk, 0, sizeof(double) * 4 * B, s));
-    NF_CUDA_TRY(cudaMemcpyAsync(lam, lambda_T, sizeof(float) * BN, cudaMemcpyDeviceToDevice, s));
     static const nf_forcing none{NF_FORCE_NONE, nullptr, nullptr, 0, 0, 0, 0, 0, 0, 0, 0};
     const nf_forcing F = g ? *g : none;
     const nf_kernel &kp = op->kp;
     const int T = 256;
     const unsigned eg = (unsigned)ceil_div((int64_t)BN, T);
+    adj_gather_kernel<<<eg, T, 0, s>>>(lambda_T, op->perm, n, B, lam);
+    NF_CUDA_TRY(cudaGetLastError());
     const int nseg = (nsteps + C - 1) / C;
     // ---- recompute segment seg forward into st, keeping every stage input (stream ss)
     auto recompute = [&](int seg, float *st, cudaStream_t ss) -> nf_status {
@@ -224,9 +244,9 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
         NF_CUDA_TRY(cudaMemcpyAsync(ubuf, ckpt + (size_t)seg * BN, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
         NF_TRY(launch_prep_g(op, ubuf, B, beta, theta, true, ss));
         NF_TRY(launch_set_clock(op, t0 + (double)s0 * dt, ss));
+        // the first stage input is the state itself; every stage kernel leaves the next one
+        NF_CUDA_TRY(cudaMemcpyAsync(st, op->U, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
         for (int j = 0; j < cnt; ++j) {
-            float *Sj = st + (size_t)j * 4 * BN;
-            NF_CUDA_TRY(cudaMemcpyAsync(Sj, ubuf, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
             for (int stage = 1; stage <= 4; ++stage) {
                 int splits = 1;
                 NF_TRY(launch_mf_pair(op, B, ss, &splits));
@@ -240,10 +260,8 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 p.ckpt = nullptr;
                 p.C = 1;
                 p.splits = splits;
+                p.stage_out = (stage < 4 || j + 1 < cnt) ? st + ((size_t)j * 4 + stage) * BN : nullptr;
                 NF_TRY(launch_stage(op, B, p, ss));
-                if (stage < 4)
-                    NF_CUDA_TRY(cudaMemcpyAsync(Sj + (size_t)stage * BN, op->U, sizeof(float) * BN,
-                                                cudaMemcpyDeviceToDevice, ss));
             }
         }
         return NF_OK;
@@ -268,13 +286,13 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
         float *const segst = stages + (size_t)bufi * seg_elems;
         // ---- reverse through the segment
         adj_prep_kernel<<<eg, T, 0, s>>>(lam, segst + ((size_t)(cnt - 1) * 4 + 3) * BN, op->q, beta, theta, n,
-                                         n_pad, B, (float)(dt / 6.0), vg);
+                                         n_pad, B, (float)(dt / 6.0), nu, gv);
         NF_CUDA_TRY(cudaGetLastError());
         for (int j = cnt - 1; j >= 0; --j) {
             for (int stg = 3; stg >= 0; --stg) {
                 float r2phys = 1.f;
                 for (int b = 0; b < B; ++b) {
-                    NF_TRY(launch_adj_sym(op, vg, B, b, wpart, gpart, &r2phys, s));
+                    NF_TRY(launch_adj_sym(op, nu, gv, B, b, wpart, gpart, &r2phys, s));
                     if (cull) NF_TRY(launch_adj_cull_reduce(op, wpart, B, b, s));
                 }
                 AdjEpiArgs ea{};
@@ -289,7 +307,10 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                                      : (j > 0 ? segst + ((size_t)(j - 1) * 4 + 3) * BN : nullptr);
                 ea.lam = lam;
                 ea.acc = acc;
-                ea.vg = vg;
+                ea.nu = nu;
+                ea.g = gv;
+                ea.perm = op->perm;
+                ea.out = (seg == 0 && j == 0 && stg == 0) ? grad_u0 : nullptr;
                 ea.q = op->q;
                 ea.beta = beta;
                 ea.theta = theta;
@@ -303,7 +324,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
         }
         NF_CUDA_TRY(cudaEventRecord(side.rev[bufi], s));  // segst may now be overwritten
     }
-    NF_CUDA_TRY(cudaMemcpyAsync(grad_u0, lam, sizeof(float) * BN, cudaMemcpyDeviceToDevice, s));
+    if (nsteps == 0) NF_CUDA_TRY(cudaMemcpyAsync(grad_u0, lambda_T, sizeof(float) * BN, cudaMemcpyDeviceToDevice, s));
     adj_finish_kernel<<<(unsigned)ceil_div(4 * B, 256), 256, 0, s>>>(gk, 4 * B, grad_kernel);
     NF_CUDA_TRY(cudaGetLastError());
     return NF_OK;

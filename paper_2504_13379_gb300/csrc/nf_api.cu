@@ -94,19 +94,13 @@ nf_status launch_nonlocal_partial(nf_operator *op, int B, cudaStream_t s, int *s
 }
 
 // ---------------------------------------------------------------- pack kernel
-// x4: coordinates as float4; xyz: coordinates times `scale` (= sqrt(log2 e) / s1) as
-// structure of arrays, so squared scaled distances are exponents of 2 for the SFU.
+// Node arrays of the dense paths, in the caller's order, zero padded.
 __global__ void pack_nodes_kernel(const float *__restrict__ x, const float *__restrict__ q, int64_t n,
-                                  int64_t n_pad, float scale, float4 *__restrict__ x4, float *__restrict__ xyz,
-                                  float *__restrict__ qp) {
+                                  int64_t n_pad, float4 *__restrict__ x4, float *__restrict__ qp) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n_pad) return;
     const bool in = j < n;
-    const float a = in ? x[3 * j] : 0.f, b = in ? x[3 * j + 1] : 0.f, c = in ? x[3 * j + 2] : 0.f;
-    x4[j] = make_float4(a, b, c, 0.f);
-    xyz[j] = a * scale;
-    xyz[n_pad + j] = b * scale;
-    xyz[2 * n_pad + j] = c * scale;
+    x4[j] = in ? make_float4(x[3 * j], x[3 * j + 1], x[3 * j + 2], 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
     qp[j] = in ? q[j] : 0.f;
 }
 
@@ -369,22 +363,20 @@ nf_status nf_operator_create(const float *x, const float *q, int64_t n, nf_kerne
         if (_e != cudaSuccess) return cleanup(cuda_fail(_e, #expr, __FILE__, __LINE__));    \
     } while (0)
     CREATE_TRY(cudaMalloc(&op->x4, op->n_pad * sizeof(float4)));
-    CREATE_TRY(cudaMalloc(&op->xyz, 3 * op->n_pad * sizeof(float)));
     CREATE_TRY(cudaMalloc(&op->q, op->n_pad * sizeof(float)));
     CREATE_TRY(cudaMalloc(&op->step_ctr, 64));
     CREATE_TRY(cudaMemsetAsync(op->step_ctr, 0, 64, s));
     op->done_ctr = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(op->step_ctr) + 16);
     op->err = reinterpret_cast<int *>(reinterpret_cast<char *>(op->step_ctr) + 32);
     op->t0_dev = reinterpret_cast<double *>(reinterpret_cast<char *>(op->step_ctr) + 40);
-    const float scale = std::sqrt(1.4426950408889634f) / kp.s1;
-    pack_nodes_kernel<<<(unsigned)ceil_div(op->n_pad, 256), 256, 0, s>>>(x, q, n, op->n_pad, scale, op->x4, op->xyz,
-                                                                         op->q);
-    CREATE_TRY(cudaGetLastError());
     if (path == NF_MATRIX_FREE) {
-        nf_status st = mf_build_row_order(op, s);
+        CREATE_TRY(cudaMalloc(&op->xyz, 3 * op->n_pad * sizeof(float)));
+        nf_status st = mf_build_nodes(op, x, q, s);
         if (st == NF_OK) st = mf_autotune(op, s);
         if (st != NF_OK) return cleanup(st);
     } else {
+        pack_nodes_kernel<<<(unsigned)ceil_div(op->n_pad, 256), 256, 0, s>>>(x, q, n, op->n_pad, op->x4, op->q);
+        CREATE_TRY(cudaGetLastError());
         const size_t entries = (size_t)op->n_pad * (size_t)op->n_pad;
         if (path == NF_DENSE_SYM_FP32) {
             CREATE_TRY(cudaMalloc(&op->W32, dense_sym_entries(op->n_pad) * sizeof(float)));
@@ -413,15 +405,14 @@ nf_status nf_operator_destroy(nf_operator *op) {
     destroy_prof_ring(op);
     cudaFree(op->x4);
     cudaFree(op->xyz);
-    cudaFree(op->rowperm);
+    cudaFree(op->perm);
+    cudaFree(op->rg);  // with rw, pc, pe, tc, te
     cudaFree(op->cull_pairs);
     cudaFree(op->cull_ptr);
     cudaFree(op->cull_slots);
-    cudaFree(op->node_blk);
     cudaFree(op->adj_pairs);
     cudaFree(op->adj_ptr);
     cudaFree(op->adj_slots);
-    cudaFree(op->adj_node_blk);
     cudaFree(op->q);
     cudaFree(op->W32);
     cudaFree(op->Whi);

@@ -194,12 +194,20 @@ struct nf_operator {
     nf_kernel kp{};
     int path = 0;
     int device = 0;
+    // Matrix-free operators keep every node array, the firing rates, the stage states and the
+    // partial sums in Hilbert order: position p holds the caller's node perm[p].  Only the
+    // elementwise kernels touch the caller's order (u, checkpoints, outputs).  Dense operators
+    // keep the caller's order (perm null).
     float4 *x4 = nullptr;    // n_pad: (x, y, z, 0)
-    float *xyz = nullptr;    // 3 x n_pad: coordinates times sqrt(log2 e)/s1, structure of arrays
+    float *xyz = nullptr;    // 3 x n_pad, structure of arrays, in the units of the kernel's exponents
+    int *perm = nullptr;     // n_pad: position -> caller's node (padding maps to itself); null: identity
+    int form = 0;            // pair form of the kernel: 0 general, 1 one Gaussian, 2-4 width ratio
+    float4 *rg = nullptr;    // node data of the symmetric kernels (SymNodes), one allocation from rg on
+    float2 *rw = nullptr;
+    float4 *pc = nullptr, *pe = nullptr, *tc = nullptr, *te = nullptr;
     int mf_variant = -1;     // launch shape of the packed pair kernel
-    int mf_sym_r = 8;        // rows per warp of the symmetric single-trajectory kernel (autotuned)
     int adj_r = 0;           // rows per warp of the adjoint pair kernel (0: not yet timed; 4 or 8)
-    int adj_blk = 0;         // its node block (0: not yet timed; 1024 or 512)
+    int adj_blk = 0;         // node block of the adjoint pair kernel (0: not yet timed; 1024 or 512)
     int mf_sched = 0;        // NF_MF_AUTO / NF_MF_SYMMETRIC / NF_MF_PACKED
     int sym_blk = 1024;      // node block of the symmetric kernel (1024, or 512 when autotuned faster)
     int planar = 0;          // every node has the same z: the symmetric kernel drops the z terms
@@ -209,11 +217,9 @@ struct nf_operator {
     int64_t cull_live = 0;
     int *cull_ptr = nullptr;     // nb + 1: each node block's live slots in cull_slots
     int *cull_slots = nullptr;   // ascending per block
-    int *node_blk = nullptr;     // n_pad: Morton block of each node
     int *adj_pairs = nullptr;    // the adjoint kernel's live pairs of 1,024-node blocks (both Gaussians)
     int64_t adj_live = 0;
-    int *adj_ptr = nullptr, *adj_slots = nullptr, *adj_node_blk = nullptr;
-    int *rowperm = nullptr;  // n_pad: row order of the packed pair kernel (Morton order of the nodes)
+    int *adj_ptr = nullptr, *adj_slots = nullptr;
     float *q = nullptr;      // n_pad, zero padded
     // dense planes (row-major, leading dimension ld = n_pad)
     float *W32 = nullptr;        // W diag(q), FP32
@@ -269,19 +275,26 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits);
 
 // matrix-free / dense nonlocal launches (g must hold q f(U) / f(U) for B trajectories)
 nf_status mf_init_attrs();
-nf_status mf_build_row_order(nf_operator *op, cudaStream_t s);
+nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaStream_t s);
 SplitPlan mf_plan(nf_operator *op);     // column splits of the multi-trajectory matrix-free launches
 int mf_splits(nf_operator *op, int B);  // partial-sum slots of a matrix-free launch over B trajectories
-int64_t sym_pair_count(const nf_operator *op);  // block pairs of the symmetric kernels
-int sym_slots(const nf_operator *op);   // node blocks of the symmetric schedule (W nu slots)
-int adj_slots(const nf_operator *op);   // node blocks of the adjoint kernel (its W nu slots)
+int mf_form(const nf_kernel &k);         // pair form of a kernel (nf_operator::form)
+float mf_unit(const nf_operator *op);    // stored coordinates per unit of the caller's
+float mf_period(const nf_operator *op);  // the kernel's period in stored coordinates (0: none)
+nf_status sym_init_attrs();
+nf_status adj_init_attrs();
+nf_status launch_sym(nf_operator *op, int B, int b_base, cudaStream_t s);
+int sym_slots(const nf_operator *op);    // node blocks of the symmetric schedule
+int64_t adj_pair_count(const nf_operator *op);  // block pairs of the adjoint kernel
+int adj_slots(const nf_operator *op);    // node blocks of the adjoint kernel (its W nu slots)
 int64_t adj_pair_capacity(const nf_operator *op);  // block pairs / slots of the adjoint kernel's
 int adj_slot_capacity(const nf_operator *op);      // smallest block (512): scratch sizes
 nf_status mf_set_cull(nf_operator *op, int enable, int64_t *live, int64_t *total, cudaStream_t s);
 nf_status launch_adj_cull_reduce(nf_operator *op, float *wpart, int B, int b, cudaStream_t s);
-nf_status launch_adj_sym(nf_operator *op, const float2 *vg, int B, int b, float *wpart, float *gpart,
+nf_status launch_adj_sym(nf_operator *op, const float *nu, const float *g, int B, int b, float *wpart, float *gpart,
                          float *r2_phys, cudaStream_t s);
-nf_status adj_autotune(nf_operator *op, const float2 *vg, int B, float *wpart, float *gpart, cudaStream_t s);
+nf_status adj_autotune(nf_operator *op, const float *nu, const float *g, int B, float *wpart, float *gpart,
+                       cudaStream_t s);
 nf_status mf_autotune(nf_operator *op, cudaStream_t s);
 void mf_launch_shape(nf_operator *op, int *R, int *TJ, int *splits);
 nf_status launch_mf_pair(nf_operator *op, int B, cudaStream_t s, int *splits_out);
@@ -312,6 +325,7 @@ struct StageParams {
     float *ckpt;
     int C;
     int splits;
+    float *stage_out;      // B x n copy of the next stage's input, in the operator's node order, or null
 };
 nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s);
 nf_status launch_set_clock(nf_operator *op, double t0, cudaStream_t s);

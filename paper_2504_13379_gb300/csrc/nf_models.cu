@@ -37,7 +37,7 @@ __device__ __forceinline__ float model_rate(const ModelArgs &m, float u, float b
 }
 
 struct ModelState {
-    float *u, *s;            // caller's state (s: depression only)
+    float *u, *s;            // caller's state (s: depression only); the rest in the operator's order
     float *U, *S;            // current stage inputs
     float *ku, *ksd;         // RK4 slope accumulators (u, s)
     float *hu, *hs;          // AB5 history: 5 slots of B x n each (u, s)
@@ -49,7 +49,13 @@ struct ModelState {
     int64_t n, n_pad;
     int B;
     const float *beta, *theta;
+    const int *perm;         // caller's node of each position (u, s), or null
 };
+
+// Index of the caller's u, s for position i of trajectory b.
+__device__ __forceinline__ int64_t caller_idx(const ModelState &st, int b, int64_t i, int64_t idx) {
+    return st.perm ? (int64_t)b * st.n + st.perm[i] : idx;
+}
 
 __device__ __forceinline__ void write_g(const ModelState &st, const ModelArgs &m, int b, int64_t i, int64_t idx,
                                         float u, float s) {
@@ -60,8 +66,7 @@ __device__ __forceinline__ void write_g(const ModelState &st, const ModelArgs &m
 }
 
 __device__ __forceinline__ float slot_sum(const ModelState &st, int b, int64_t i) {
-    float I = 0.f;
-    for (int sp = 0; sp < st.splits; ++sp) I += st.partial[((int64_t)sp * st.B + b) * st.n_pad + i];
+    const float I = sum_slots(st.partial + (int64_t)b * st.n_pad + i, (int64_t)st.B * st.n_pad, st.splits);
     return st.rs ? I * st.rs[i] : I;
 }
 
@@ -71,8 +76,9 @@ __global__ void model_prep_kernel(ModelState st, ModelArgs m) {
     if (idx >= (int64_t)st.B * st.n) return;
     const int b = (int)(idx / st.n);
     const int64_t i = idx - (int64_t)b * st.n;
-    const float u = st.u[idx];
-    const float s = (m.kind == NF_MODEL_DEPRESSION) ? st.s[idx] : 1.f;
+    const int64_t ci = caller_idx(st, b, i, idx);
+    const float u = st.u[ci];
+    const float s = (m.kind == NF_MODEL_DEPRESSION) ? st.s[ci] : 1.f;
     st.U[idx] = u;
     if (m.kind == NF_MODEL_DEPRESSION) st.S[idx] = s;
     write_g(st, m, b, i, idx, u, s);
@@ -95,7 +101,8 @@ __global__ void model_rk4_stage_kernel(ModelState st, ModelArgs m, int stage, fl
         if (dep) st.hs[h] = ks;
     }
     float Un, Sn = 1.f;
-    const float uv = st.u[idx], sv = dep ? st.s[idx] : 1.f;
+    const int64_t ci = caller_idx(st, b, i, idx);
+    const float uv = st.u[ci], sv = dep ? st.s[ci] : 1.f;
     if (stage == 1) {
         st.ku[idx] = ku;
         Un = fmaf(0.5f * dt, ku, uv);
@@ -113,10 +120,10 @@ __global__ void model_rk4_stage_kernel(ModelState st, ModelArgs m, int stage, fl
         }
     } else {
         Un = fmaf(dt / 6.f, st.ku[idx] + ku, uv);
-        st.u[idx] = Un;
+        st.u[ci] = Un;
         if (dep) {
             Sn = fmaf(dt / 6.f, st.ksd[idx] + ks, sv);
-            st.s[idx] = Sn;
+            st.s[ci] = Sn;
         }
     }
     st.U[idx] = Un;
@@ -133,7 +140,8 @@ __global__ void model_ab5_kernel(ModelState st, ModelArgs m, int step, float dt)
     const int64_t i = idx - (int64_t)b * st.n;
     const bool dep = m.kind == NF_MODEL_DEPRESSION;
     const int64_t plane = (int64_t)st.B * st.n;
-    const float uv = st.u[idx], sv = dep ? st.s[idx] : 1.f;
+    const int64_t ci = caller_idx(st, b, i, idx);
+    const float uv = st.u[ci], sv = dep ? st.s[ci] : 1.f;
     const float Fu = -uv + slot_sum(st, b, i);
     const float Fs = dep ? (1.f - sv - m.beta_d * sv * model_rate(m, uv, st.beta[b], st.theta[b])) * m.tau_inv : 0.f;
     st.hu[(int64_t)(step % 5) * plane + idx] = Fu;
@@ -147,11 +155,11 @@ __global__ void model_ab5_kernel(ModelState st, ModelArgs m, int step, float dt)
         if (dep) ds = fmaf(c[k], st.hs[h], ds);
     }
     const float un = fmaf(dt, du, uv);
-    st.u[idx] = un;
+    st.u[ci] = un;
     float sn = 1.f;
     if (dep) {
         sn = fmaf(dt, ds, sv);
-        st.s[idx] = sn;
+        st.s[ci] = sn;
     }
     write_g(st, m, b, i, idx, un, sn);
 }
@@ -204,6 +212,7 @@ extern "C" nf_status nf_field_advance(nf_operator *op, const nf_model *model, in
     st.B = B;
     st.beta = beta;
     st.theta = theta;
+    st.perm = op->perm;
     ModelArgs m{};
     m.kind = model->kind;
     m.rate = model->rate;
