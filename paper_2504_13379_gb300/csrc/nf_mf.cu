@@ -903,6 +903,21 @@ nf_status launch_reduce_I(nf_operator *op, int B, int splits, float *I, cudaStre
 }
 
 // ----------------------------------------------------------------------------
+// Constants of the flat manufactured forcing (host side of forcing_value): per Gaussian of the
+// kernel with amplitude A and width w, p = 1 / w^2.
+struct FlatTerm {
+    double amp;        // +-A / (2 pi sigma^2)
+    double rs, prs;    // r / (p + r), -p r / (p + r)
+    double k;          // sqrt(p + r)
+    double half_root;  // sqrt(pi / (p + r)) / 2
+};
+struct FlatConst {
+    double L, iL, r, norm;  // period, 1 / (2 sigma^2), 1 / (2 pi sigma^2)
+    double c0;              // the convolution's constant part
+    FlatTerm t[2];
+    int terms;
+};
+
 // Fused RK4 stage: I = sum of splits; k_s = -U_s + I + gamma(t_s); RK4 bookkeeping;
 // next stage input and its g.  On the last stage the last block advances the
 // device step counter, so one captured step can be replayed.
@@ -916,8 +931,8 @@ struct StageKArgs {
     const float *rs;    // BF16X2 row scale, or null
     const float *beta, *theta;
     nf_forcing F;
-    const float4 *x4;   // node coordinates (the flat manufactured forcing)
-    nf_kernel kp;
+    FlatConst fc;       // flat manufactured forcing
+    const float4 *x4;   // node coordinates (manufactured forcings)
     const double *t0;
     double dt;
     int stage;
@@ -938,46 +953,45 @@ struct StageKArgs {
 //   int_{d0}^{d1} exp(-p d^2 - r (d - a')^2) dd
 //     = exp(-p r a'^2 / (p + r)) (1/2) sqrt(pi / (p + r)) [erf(k (d1 - m)) - erf(k (d0 - m))],
 // r = 1 / (2 sigma^2), m = r a' / (p + r), k = sqrt(p + r).
+// The forcing is FP64 arithmetic on a chip whose FP64 pipe gives two lanes per clock per SM, so
+// what does not depend on the node is taken out: constants come from the host, cos t and sin t
+// from one thread per block, an erf is evaluated only where it is not +-1 to the last bit, and a
+// piece whose two erf agree is 0 without its exponential (all pieces but one, away from the
+// kink lines).
 constexpr double kPi = 3.14159265358979323846;
-__device__ __forceinline__ double gauss_piece(double p, double r, double a, double d0, double d1) {
-    const double s = p + r, m = r * a / s, k = sqrt(s);
-    return exp(-p * r * a * a / s) * 0.5 * sqrt(kPi / s) * (erf(k * (d1 - m)) - erf(k * (d0 - m)));
+__device__ __forceinline__ double erf_sat(double z) { return z >= 6.0 ? 1.0 : (z <= -6.0 ? -1.0 : erf(z)); }
+__device__ __forceinline__ double gauss_piece(const FlatTerm &g, double a, double d0, double d1) {
+    const double m = g.rs * a, diff = erf_sat(g.k * (d1 - m)) - erf_sat(g.k * (d0 - m));
+    return diff == 0.0 ? 0.0 : exp(g.prs * a * a) * g.half_root * diff;
 }
-__device__ __forceinline__ double flat_factor(double a, double p, double r, double L) {
+__device__ __forceinline__ double flat_factor(const FlatTerm &g, double a, double L) {
     const double h = 0.5 * L;
-    if (a >= 0.0) return gauss_piece(p, r, a - L, -h, a - h) + gauss_piece(p, r, a, a - h, h);
-    return gauss_piece(p, r, a, -h, a + h) + gauss_piece(p, r, a + L, a + h, h);
+    if (a >= 0.0) return gauss_piece(g, a - L, -h, a - h) + gauss_piece(g, a, a - h, h);
+    return gauss_piece(g, a, -h, a + h) + gauss_piece(g, a + L, a + h, h);
 }
-__device__ __forceinline__ double nearest_image(double d, double L) { return d - L * rint(d / L); }
 
-// i: position in the operator's order (x4); node: the caller's index (Y1, Y2)
-__device__ __forceinline__ double forcing_value(const nf_forcing &F, const float4 *x4, const nf_kernel &kp,
-                                                int64_t i, int64_t node, double t, float beta, float theta) {
+// i: position in the operator's order (x4); node: the caller's index (Y1, Y2); ct, sn = cos t, sin t
+__device__ __forceinline__ double forcing_value(const nf_forcing &F, const FlatConst &fc, const float4 *x4, int64_t i,
+                                                int64_t node, double ct, double sn, float beta, float theta) {
     if (F.kind == NF_FORCE_MMS_FLAT) {
         // z = G(x, x0(t); sigma) + c on the periodic square; gamma = du*/dt + u* - scale C,
         // C = int_cell w(dist(x, y)) z(y) dy: the constant part integrates w over the
         // displacement square, the Gaussian part is separable (flat_factor per coordinate)
-        const double L = kp.period, sg = F.sigma, r = 1.0 / (2.0 * sg * sg);
-        const double x0 = F.radius * cos(t), y0 = F.radius * sin(t);
+        const double x0 = F.radius * ct, y0 = F.radius * sn;
         const float4 xi = x4[i];
-        const double ax = nearest_image((double)xi.x - x0, L), ay = nearest_image((double)xi.y - y0, L);
-        const double G = exp(-(ax * ax + ay * ay) * r) / (2.0 * kPi * sg * sg);
+        double ax = (double)xi.x - x0, ay = (double)xi.y - y0;
+        ax -= fc.L * rint(ax * fc.iL);
+        ay -= fc.L * rint(ay * fc.iL);
+        const double G = exp(-(ax * ax + ay * ay) * fc.r) * fc.norm;
         const double z = G + F.c;
-        const double dz = G * (ax * (-F.radius * sin(t)) + ay * (F.radius * cos(t))) / (sg * sg);
+        const double dz = G * (ay * x0 - ax * y0) * (2.0 * fc.r);
         const double us = (double)theta + log(z / (1.0 - z)) / (double)beta;
         const double dus = dz / ((double)beta * z * (1.0 - z));
-        const double amp[2] = {(double)kp.A1, -(double)kp.A2}, wid[2] = {(double)kp.s1, (double)kp.s2};
-        double C = 0.0;
-        for (int h = 0; h < 2; ++h) {
-            if (amp[h] == 0.0) continue;
-            const double p = 1.0 / (wid[h] * wid[h]);
-            const double e = sqrt(kPi) * wid[h] * erf(0.5 * L / wid[h]);
-            C += amp[h] * (F.c * e * e + flat_factor(ax, p, r, L) * flat_factor(ay, p, r, L) /
-                                             (2.0 * kPi * sg * sg));
-        }
+        double C = fc.c0;
+        for (int h = 0; h < fc.terms; ++h)
+            C += fc.t[h].amp * (flat_factor(fc.t[h], ax, fc.L) * flat_factor(fc.t[h], ay, fc.L));
         return dus + us - F.scale * C;
     }
-    if (F.kind != NF_FORCE_MMS_EIGEN && F.kind != NF_FORCE_MMS_SPHERE) return 0.0;
     double Y1, Y2;
     if (F.kind == NF_FORCE_MMS_SPHERE) {  // Y1 = z / 2 (degree 1), Y2 = x y (degree 2) at the node
         const float4 xi = x4[i];
@@ -988,7 +1002,7 @@ __device__ __forceinline__ double forcing_value(const nf_forcing &F, const float
         Y2 = F.Y2[node];
     }
     const double Y = Y1 + Y2;
-    const double a = F.a0 * cos(t), da = -F.a0 * sin(t);
+    const double a = F.a0 * ct, da = -F.a0 * sn;
     const double z = F.c + a * Y;
     const double us = (double)theta + log(z / (1.0 - z)) / (double)beta;
     const double dus = da * Y / ((double)beta * z * (1.0 - z));
@@ -998,16 +1012,25 @@ __device__ __forceinline__ double forcing_value(const nf_forcing &F, const float
 __global__ void rk4_stage_kernel(StageKArgs a) {
     const long long step = *a.step_ctr;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double time_cs[2];  // cos t, sin t of the stage
+    if (a.F.kind != NF_FORCE_NONE) {
+        if (threadIdx.x == 0) {
+            const double cs = (a.stage == 1) ? 0.0 : (a.stage == 4 ? 1.0 : 0.5);
+            const double ts = *a.t0 + (double)step * a.dt + cs * a.dt;
+            sincos(ts, &time_cs[1], &time_cs[0]);
+        }
+        __syncthreads();
+    }
     if (idx < (int64_t)a.B * a.n) {
         const int b = (int)(idx / a.n);
         const int64_t i = idx - (int64_t)b * a.n;
         float I = sum_slots(a.partial + (int64_t)b * a.n_pad + i, (int64_t)a.B * a.n_pad, a.splits);
         if (a.rs) I *= a.rs[i];
-        const double cs = (a.stage == 1) ? 0.0 : (a.stage == 4 ? 1.0 : 0.5);
-        const double ts = *a.t0 + (double)step * a.dt + cs * a.dt;
         const float bb = a.beta[b], th = a.theta[b];
         const int64_t node = a.perm ? a.perm[i] : i, cidx = (int64_t)b * a.n + node;
-        const float gam = (float)forcing_value(a.F, a.x4, a.kp, i, node, ts, bb, th);
+        const float gam = a.F.kind == NF_FORCE_NONE
+                              ? 0.f
+                              : (float)forcing_value(a.F, a.fc, a.x4, i, node, time_cs[0], time_cs[1], bb, th);
         const float Uv = a.U[idx], uv = a.u[cidx];
         const float k = (-Uv + I) + gam;
         const float dt = (float)a.dt;
@@ -1060,6 +1083,24 @@ nf_status launch_set_clock(nf_operator *op, double t0, cudaStream_t s) {
     return NF_OK;
 }
 
+static FlatConst flat_const(const nf_forcing &F, const nf_kernel &kp) {
+    FlatConst c{};
+    const double sg2 = F.sigma * F.sigma;
+    c.L = kp.period;
+    c.iL = 1.0 / c.L;
+    c.r = 1.0 / (2.0 * sg2);
+    c.norm = 1.0 / (2.0 * kPi * sg2);
+    const double amp[2] = {(double)kp.A1, -(double)kp.A2}, wid[2] = {(double)kp.s1, (double)kp.s2};
+    for (int h = 0; h < 2; ++h) {
+        if (amp[h] == 0.0) continue;
+        const double p = 1.0 / (wid[h] * wid[h]), s = p + c.r;
+        const double e = std::sqrt(kPi) * wid[h] * std::erf(0.5 * c.L / wid[h]);
+        c.c0 += amp[h] * F.c * e * e;
+        c.t[c.terms++] = FlatTerm{amp[h] * c.norm, c.r / s, -p * c.r / s, std::sqrt(s), 0.5 * std::sqrt(kPi / s)};
+    }
+    return c;
+}
+
 nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s) {
     StageKArgs a{};
     a.partial = op->partial;
@@ -1076,8 +1117,8 @@ nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_
     a.beta = p.beta;
     a.theta = p.theta;
     a.F = p.forcing;
+    if (a.F.kind == NF_FORCE_MMS_FLAT) a.fc = flat_const(a.F, op->kp);
     a.x4 = op->x4;
-    a.kp = op->kp;
     a.t0 = op->t0_dev;
     a.dt = p.dt;
     a.stage = p.stage;
