@@ -55,8 +55,8 @@ def build(force: bool = False, verbose: bool = False, ptxas_v: bool = False) -> 
     def compile_one(src):
         obj = os.path.join(OBJ, os.path.basename(src) + ".o")
         # FP64 setup (stencils, RBF-QF solves) rounds every operation separately, like a
-        # plain IEEE evaluation without fused multiply-add.
-        per_file = ["-fmad=false"] if os.path.basename(src) == "nf_setup.cu" else []
+        # plain IEEE evaluation, except where it calls fma itself.
+        per_file = ["-fmad=false"] if os.path.basename(src) in ("nf_setup.cu", "nf_quad.cu") else []
         cmd = [cc, *ARCH, *NVCC_FLAGS, *per_file, *extra, "-I", INCLUDE, "-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:

@@ -231,6 +231,7 @@ struct nf_operator {
     size_t partial_cap = 0;
     float *g = nullptr;          // [B][n_pad]: q_j f(U_j) (matrix-free) or f(U_j) (dense)
     float *U = nullptr;          // [B][n]: current stage input
+    float *us = nullptr;         // [B][n]: the state in the operator's order (perm operators)
     float *ks = nullptr;         // [B][n]: RK4 slope accumulator
     size_t state_cap = 0;        // elements of U / ks
     size_t g_cap = 0;
@@ -270,6 +271,10 @@ struct SplitPlan {
 };
 SplitPlan plan_splits(int64_t n_pad, int rows_per_block, int tile_cols, int resident_blocks_per_sm,
                       int max_splits = 64);
+
+// setup helpers (nf_setup.cu): *flag <- 1 if an index lies outside [0, n); exclusive scan, out[len] = total
+void launch_validate_indices(const int32_t *idx, int64_t cnt, int64_t n, int *flag, cudaStream_t s);
+void launch_exclusive_scan(const int32_t *in, int64_t len, int32_t *out, cudaStream_t s);
 
 nf_status ensure_workspace(nf_operator *op, int B, int splits);
 
