@@ -237,10 +237,11 @@ NF_API nf_status nf_operator_launch_shape(nf_operator *op, int *rows_per_warp, i
 /* Schedule of a matrix-free operator's sums for up to three trajectories (Eq. (2.9); from
  * four trajectories on the multi-trajectory kernels share each pair's exponentials):
  *   NF_MF_AUTO       the symmetric block-pair kernel (each unordered pair once, w radial)
- *                    when it has block pairs for 2/3 of the SMs and its partial sums
- *                    (4 n^2 / 1024 bytes per trajectory) fit an eighth of the device
- *                    memory, else the packed kernel (default; the switch is at about
- *                    13,300 nodes on 152 SMs, and again at about 3 million);
+ *                    above 3,072 nodes, on blocks of 256 nodes below about 13,300 nodes, while
+ *                    its partial sums (4 n^2 / 1024 bytes per trajectory) fit an eighth of the
+ *                    device memory (to about 3 million nodes), else the packed kernel; up to
+ *                    3,072 nodes the packed kernel with the RK4 stage in the same launch
+ *                    (default);
  *   NF_MF_SYMMETRIC  always the symmetric kernel;
  *   NF_MF_PACKED     always the packed row-block x column-split kernel (ordered pairs);
  *   NF_MF_SYMMETRIC_512, NF_MF_SYMMETRIC_1024   the symmetric kernel with that node-block

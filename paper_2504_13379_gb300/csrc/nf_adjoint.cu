@@ -205,7 +205,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
     // pairs, and each node's live W nu slots are added into slot 0 before the epilogue
     const bool cull = op->mf_cull && op->adj_pairs;
     const int Cseg = std::min(C, std::max(nsteps, 1));
-    float *stages = nullptr, *lam = nullptr, *acc = nullptr, *ubuf = nullptr, *wpart = nullptr, *gpart = nullptr;
+    float *stages = nullptr, *lam = nullptr, *acc = nullptr, *wpart = nullptr, *gpart = nullptr;
     float *nu = nullptr;
     double *gk = nullptr;
     StreamScratch scratch(s);  // freed (stream-ordered) on every return below
@@ -215,7 +215,6 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
     NF_CUDA_TRY(scratch.alloc(&stages, sizeof(float) * 2 * seg_elems));
     NF_CUDA_TRY(scratch.alloc(&lam, sizeof(float) * BN));
     NF_CUDA_TRY(scratch.alloc(&acc, sizeof(float) * BN));
-    NF_CUDA_TRY(scratch.alloc(&ubuf, sizeof(float) * BN));
     // W nu slots and parameter partials for the smallest node block the kernel may take
     NF_CUDA_TRY(scratch.alloc(&wpart, sizeof(float) * (size_t)adj_slot_capacity(op) * B * n_pad));
     NF_CUDA_TRY(scratch.alloc(&gpart, sizeof(float) * 4 * (size_t)B * adj_pair_capacity(op)));
@@ -241,8 +240,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
     auto recompute = [&](int seg, float *st, cudaStream_t ss) -> nf_status {
         const int s0 = seg * C;
         const int cnt = std::min(C, nsteps - s0);
-        NF_CUDA_TRY(cudaMemcpyAsync(ubuf, ckpt + (size_t)seg * BN, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
-        NF_TRY(launch_prep_g(op, ubuf, B, beta, theta, true, ss));
+        NF_TRY(launch_prep_g(op, ckpt + (size_t)seg * BN, B, beta, theta, true, ss));
         NF_TRY(launch_set_clock(op, t0 + (double)s0 * dt, ss));
         // the first stage input is the state itself; every stage kernel leaves the next one
         NF_CUDA_TRY(cudaMemcpyAsync(st, op->U, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
@@ -251,7 +249,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 int splits = 1;
                 NF_TRY(launch_mf_pair(op, B, ss, &splits));
                 StageParams p{};
-                p.u = ubuf;
+                p.u = nullptr;  // the state advances inside the operator only
                 p.beta = beta;
                 p.theta = theta;
                 p.forcing = F;
@@ -260,6 +258,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 p.ckpt = nullptr;
                 p.C = 1;
                 p.splits = splits;
+                p.overlap = true;
                 p.stage_out = (stage < 4 || j + 1 < cnt) ? st + ((size_t)j * 4 + stage) * BN : nullptr;
                 NF_TRY(launch_stage(op, B, p, ss));
             }

@@ -50,7 +50,7 @@ int num_sms() {
 // ---------------------------------------------------------------- workspace
 nf_status ensure_workspace(nf_operator *op, int B, int splits) {
     const size_t need_p = (size_t)splits * B * op->n_pad;
-    const size_t need_g = (size_t)B * op->n_pad;
+    const size_t need_g = (fused_fits(op, B) ? 2 : 1) * (size_t)B * op->n_pad;  // fused stages alternate
     const size_t need_s = (size_t)B * op->n;
     // captured graphs hold workspace pointers: drop them before anything moves
     if (need_p > op->partial_cap || need_g > op->g_cap || need_s > op->state_cap) destroy_graphs(op);
@@ -72,8 +72,10 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits) {
     if (need_s > op->state_cap) {
         if (op->U) NF_CUDA_TRY(cudaFree(op->U));
         if (op->ks) NF_CUDA_TRY(cudaFree(op->ks));
-        op->U = op->ks = nullptr;
+        if (op->us) NF_CUDA_TRY(cudaFree(op->us));
+        op->U = op->ks = op->us = nullptr;
         op->state_cap = 0;
+        if (op->perm) NF_CUDA_TRY(cudaMalloc(&op->us, need_s * sizeof(float)));
         NF_CUDA_TRY(cudaMalloc(&op->U, need_s * sizeof(float)));
         NF_CUDA_TRY(cudaMalloc(&op->ks, need_s * sizeof(float)));
         op->state_cap = need_s;
@@ -191,15 +193,6 @@ static nf_status rk4_step_graph(nf_operator *op, float *u, int B, double dt, con
             }
             continue;
         }
-        st = launch_nonlocal_partial(op, B, cs, &splits);
-        if (st != NF_OK) break;
-        if (op->profile) {
-            cudaError_t pe = cudaEventRecordWithFlags(op->prof_ring[2 * (stage - 1) + 1], cs, cudaEventRecordExternal);
-            if (pe != cudaSuccess) {
-                st = cuda_fail(pe, "cudaEventRecord", __FILE__, __LINE__);
-                break;
-            }
-        }
         StageParams p{};
         p.u = u;
         p.beta = beta;
@@ -209,6 +202,19 @@ static nf_status rk4_step_graph(nf_operator *op, float *u, int B, double dt, con
         p.stage = stage;
         p.ckpt = ckpt;
         p.C = C;
+        p.overlap = !op->profile;
+        // forced stages keep their own launch: the forcing's FP64 work wants full warps
+        const bool fused = fused_fits(op, B) && F.kind == NF_FORCE_NONE;
+        st = fused ? fused_stage(op, B, p, cs) : launch_nonlocal_partial(op, B, cs, &splits);
+        if (st != NF_OK) break;
+        if (op->profile) {
+            cudaError_t pe = cudaEventRecordWithFlags(op->prof_ring[2 * (stage - 1) + 1], cs, cudaEventRecordExternal);
+            if (pe != cudaSuccess) {
+                st = cuda_fail(pe, "cudaEventRecord", __FILE__, __LINE__);
+                break;
+            }
+        }
+        if (fused) continue;
         p.splits = splits;
         st = launch_stage(op, B, p, cs);
     }
@@ -422,6 +428,7 @@ nf_status nf_operator_destroy(nf_operator *op) {
     cudaFree(op->g);
     cudaFree(op->U);
     cudaFree(op->ks);
+    cudaFree(op->us);
     cudaFree(op->step_ctr);
     delete op;
     return NF_OK;
@@ -454,6 +461,7 @@ nf_status nf_nonlocal_apply(nf_operator *op, const float *u, int B, const float 
     }
     NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B)));
     NF_TRY(launch_prep_g(op, u, B, beta, theta, false, s));
+    if (fused_fits(op, B)) return fused_apply(op, B, I, s);
     int splits = 1;
     NF_TRY(launch_nonlocal_partial(op, B, s, &splits));
     NF_TRY(launch_reduce_I(op, B, splits, I, s));

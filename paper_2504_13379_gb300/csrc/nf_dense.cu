@@ -21,7 +21,7 @@
 //                    own s_i): the precision form of the symmetric operator.
 // Work items (32-row block, column split) write partial sums like the matrix-free
 // kernel, so the same stage kernel finishes the RK4 step.
-#include "nf_internal.cuh"
+#include "nf_pairs.cuh"
 
 #include <algorithm>
 
@@ -111,19 +111,11 @@ constexpr int SB = 1024;
 constexpr int SYM_THREADS = 256;
 constexpr int SYM_WARPS = SYM_THREADS / 32;
 
-__device__ __forceinline__ void sym_block_pair(int64_t t, int &I, int &J) {
-    int64_t j = (int64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-    while (j * (j + 1) / 2 > t) --j;
-    while ((j + 1) * (j + 2) / 2 <= t) ++j;
-    J = (int)j;
-    I = (int)(t - j * (j + 1) / 2);
-}
-
 // grid (pairs, SB / 16): each block writes 16 rows of one block pair
 __global__ void dense_build_sym_kernel(const float4 *__restrict__ x4, float A1, float is1, float A2, float is2,
                                        float per, float ip, float *__restrict__ K) {
     int I, J;
-    sym_block_pair(blockIdx.x, I, J);
+    sym_pair(blockIdx.x, I, J);
     float *blk = K + (int64_t)blockIdx.x * SB * SB;
     for (int rr = 0; rr < 16; ++rr) {
         const int r = blockIdx.y * 16 + rr;
@@ -176,7 +168,7 @@ __global__ void dense_build_sym_bf16x2_kernel(const float4 *__restrict__ x4, con
                                               float A1, float is1, float A2, float is2, float per, float ip,
                                               uint4 *__restrict__ K) {
     int I, J;
-    sym_block_pair(blockIdx.x, I, J);
+    sym_pair(blockIdx.x, I, J);
     uint4 *blk = K + (int64_t)blockIdx.x * SB * SBC * 2;
     for (int rr = 0; rr < 16; ++rr) {
         const int r = blockIdx.y * 16 + rr;
@@ -354,7 +346,7 @@ gemv_sym_fp32_kernel(const float *__restrict__ K, const float *__restrict__ g_al
     __shared__ __align__(16) float colred[SYM_WARPS][SB];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int I, J;
-    sym_block_pair(blockIdx.x, I, J);
+    sym_pair(blockIdx.x, I, J);
     const bool diag = I == J;
     const float *g = g_all + (int64_t)b * n_pad;
     for (int k = tid; k < SB; k += SYM_THREADS) {
@@ -442,7 +434,7 @@ gemv_sym_bf16x2_kernel(const uint4 *__restrict__ K, const float *__restrict__ g_
     __shared__ __align__(16) float colred[SYM_WARPS][SB];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int I, J;
-    sym_block_pair(blockIdx.x, I, J);
+    sym_pair(blockIdx.x, I, J);
     const bool diag = I == J;
     const float *g = g_all + (int64_t)b * n_pad;
     for (int k = tid; k < SB; k += SYM_THREADS) {

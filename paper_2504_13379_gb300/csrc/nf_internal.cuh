@@ -164,6 +164,32 @@ __device__ __forceinline__ float sum_slots(const float *__restrict__ base, int64
     return s;
 }
 
+// Programmatic dependent launch: a kernel launched with launch_dependent may start while the kernel
+// before it in the stream still runs.  Every thread calls pdl_wait() before it touches
+// anything that earlier work in the stream writes (it returns once that work is complete and
+// visible; at once in a normal launch), and every path of such a kernel calls it, so a kernel's
+// completion implies that of everything before it.  pdl_trigger() lets the next kernel start;
+// called after pdl_wait(), it also lets that kernel read, before its own pdl_wait(), what was
+// written up to two kernels earlier.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, bool overlap,
+                             A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -331,8 +357,14 @@ struct StageParams {
     int C;
     int splits;
     float *stage_out;      // B x n copy of the next stage's input, in the operator's node order, or null
+    bool overlap;          // the kernel before is the pair kernel: start while it runs (pdl_wait)
 };
 nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s);
+// One launch per sum on small matrix-free node sets: pair sums with the RK4 stage (fused_stage) or
+// the output (fused_apply) in the same kernel.
+bool fused_fits(const nf_operator *op, int B);
+nf_status fused_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s);
+nf_status fused_apply(nf_operator *op, int B, float *I, cudaStream_t s);
 nf_status launch_set_clock(nf_operator *op, double t0, cudaStream_t s);
 
 // nonlocal sum of the current g into partial (path dispatch)

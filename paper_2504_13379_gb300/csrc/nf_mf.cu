@@ -154,6 +154,174 @@ mf_pair_kernel(const float4 *__restrict__ x4, const float *__restrict__ g, int64
 }
 
 // ----------------------------------------------------------------------------
+// RK4 stage of one node, shared by the stage kernel and the fused small-set kernel.
+__device__ __forceinline__ float firing_rate(float u, float beta, float theta) {
+    return 1.0f / (1.0f + expf(-beta * (u - theta)));
+}
+
+// Constants of the flat manufactured forcing (host side of forcing_value): per Gaussian of the
+// kernel with amplitude A and width w, p = 1 / w^2.
+struct FlatTerm {
+    double amp;        // +-A / (2 pi sigma^2)
+    double rs, prs;    // r / (p + r), -p r / (p + r)
+    double k;          // sqrt(p + r)
+    double half_root;  // sqrt(pi / (p + r)) / 2
+};
+struct FlatConst {
+    double L, iL, r, norm;  // period, 1 / (2 sigma^2), 1 / (2 pi sigma^2)
+    double c0;              // the convolution's constant part
+    FlatTerm t[2];
+    int terms;
+};
+
+// Fused RK4 stage: I = sum of splits; k_s = -U_s + I + gamma(t_s); RK4 bookkeeping;
+// next stage input and its g.  On the last stage the last block advances the
+// device step counter, so one captured step can be replayed.
+struct StageKArgs {
+    const float *partial;
+    int splits;
+    int64_t n, n_pad;
+    int B;
+    float *u;           // caller's state, written by stage 4 (null: kept inside only)
+    float *us;          // the state in the operator's order: u itself without perm
+    float *U, *ks, *g;
+    const float *q;     // matrix-free: g = q f; dense: g = f (q lives in W)
+    const float *rs;    // BF16X2 row scale, or null
+    const float *beta, *theta;
+    nf_forcing F;
+    FlatConst fc;       // flat manufactured forcing
+    const float4 *x4;   // node coordinates (manufactured forcings)
+    const double *t0;
+    double dt;
+    int stage;
+    long long *step_ctr;
+    unsigned *done_ctr;
+    float *ckpt;
+    int C;
+    const int *perm;    // caller's node of each position (u, ckpt, Y1, Y2), or null
+    float *stage_out;   // next stage's input, kept by the adjoint's recomputation, or null
+    int *err;           // operator's device flag: DEV_NONFINITE on a non-finite new state
+};
+
+// Flat manufactured forcing (NF_FORCE_MMS_FLAT).  One factor of the convolution term:
+//   J(a) = int_{-L/2}^{L/2} exp(-p d^2) exp(-e(d)^2 / (2 sigma^2)) dd,  e(d) = nearest image of a - d,
+// a = nearest image of x - x0 in one coordinate.  e(d) = a - d except past the point where
+// a - d leaves [-L/2, L/2] (d < a - L/2 for a >= 0, d > a + L/2 for a < 0), where it is
+// a - d -+ L.  Each piece is a Gaussian product integrated in closed form:
+//   int_{d0}^{d1} exp(-p d^2 - r (d - a')^2) dd
+//     = exp(-p r a'^2 / (p + r)) (1/2) sqrt(pi / (p + r)) [erf(k (d1 - m)) - erf(k (d0 - m))],
+// r = 1 / (2 sigma^2), m = r a' / (p + r), k = sqrt(p + r).
+// The forcing is FP64 arithmetic on a chip whose FP64 pipe gives two lanes per clock per SM, so
+// what does not depend on the node is taken out: constants come from the host, cos t and sin t
+// from one thread per block, an erf is evaluated only where it is not +-1 to the last bit, and a
+// piece whose two erf agree is 0 without its exponential (all pieces but one, away from the
+// kink lines).
+constexpr double kPi = 3.14159265358979323846;
+__device__ __forceinline__ double erf_sat(double z) { return z >= 6.0 ? 1.0 : (z <= -6.0 ? -1.0 : erf(z)); }
+__device__ __forceinline__ double gauss_piece(const FlatTerm &g, double a, double d0, double d1) {
+    const double m = g.rs * a, diff = erf_sat(g.k * (d1 - m)) - erf_sat(g.k * (d0 - m));
+    return diff == 0.0 ? 0.0 : exp(g.prs * a * a) * g.half_root * diff;
+}
+__device__ __forceinline__ double flat_factor(const FlatTerm &g, double a, double L) {
+    const double h = 0.5 * L;
+    if (a >= 0.0) return gauss_piece(g, a - L, -h, a - h) + gauss_piece(g, a, a - h, h);
+    return gauss_piece(g, a, -h, a + h) + gauss_piece(g, a + L, a + h, h);
+}
+
+// i: position in the operator's order (x4); node: the caller's index (Y1, Y2); ct, sn = cos t, sin t
+__device__ __forceinline__ double forcing_value(const nf_forcing &F, const FlatConst &fc, const float4 *x4, int64_t i,
+                                                int64_t node, double ct, double sn, float beta, float theta) {
+    if (F.kind == NF_FORCE_MMS_FLAT) {
+        // z = G(x, x0(t); sigma) + c on the periodic square; gamma = du*/dt + u* - scale C,
+        // C = int_cell w(dist(x, y)) z(y) dy: the constant part integrates w over the
+        // displacement square, the Gaussian part is separable (flat_factor per coordinate)
+        const double x0 = F.radius * ct, y0 = F.radius * sn;
+        const float4 xi = x4[i];
+        double ax = (double)xi.x - x0, ay = (double)xi.y - y0;
+        ax -= fc.L * rint(ax * fc.iL);
+        ay -= fc.L * rint(ay * fc.iL);
+        const double G = exp(-(ax * ax + ay * ay) * fc.r) * fc.norm;
+        const double z = G + F.c;
+        const double dz = G * (ay * x0 - ax * y0) * (2.0 * fc.r);
+        const double us = (double)theta + log(z / (1.0 - z)) / (double)beta;
+        const double dus = dz / ((double)beta * z * (1.0 - z));
+        double C = fc.c0;
+        for (int h = 0; h < fc.terms; ++h)
+            C += fc.t[h].amp * (flat_factor(fc.t[h], ax, fc.L) * flat_factor(fc.t[h], ay, fc.L));
+        return dus + us - F.scale * C;
+    }
+    double Y1, Y2;
+    if (F.kind == NF_FORCE_MMS_SPHERE) {  // Y1 = z / 2 (degree 1), Y2 = x y (degree 2) at the node
+        const float4 xi = x4[i];
+        Y1 = 0.5 * (double)xi.z;
+        Y2 = (double)xi.x * (double)xi.y;
+    } else {
+        Y1 = F.Y1[node];
+        Y2 = F.Y2[node];
+    }
+    const double Y = Y1 + Y2;
+    const double a = F.a0 * ct, da = -F.a0 * sn;
+    const double z = F.c + a * Y;
+    const double us = (double)theta + log(z / (1.0 - z)) / (double)beta;
+    const double dus = da * Y / ((double)beta * z * (1.0 - z));
+    return dus + us - (F.lam0 * F.c + a * (F.lam1 * Y1 + F.lam2 * Y2));
+}
+
+// The tableau update of one node from its sum I: k_s = -U_s + I + gamma, the RK4 bookkeeping, the
+// next stage's input and its g (g_out: where the next sum reads it).
+struct StageNode {
+    float Uv, uv, ksv, bb, th, qv;  // U_s, u, slope accumulator, beta, theta, q
+    int64_t node;                   // the caller's index
+};
+__device__ __forceinline__ StageNode stage_load(const StageKArgs &a, int b, int64_t i, int64_t idx) {
+    return StageNode{a.U[idx], a.us[idx], a.stage > 1 ? a.ks[idx] : 0.f, a.beta[b], a.theta[b],
+                     a.q ? a.q[i] : 1.f, a.perm ? (int64_t)a.perm[i] : i};
+}
+__device__ __forceinline__ void stage_update(const StageKArgs &a, const StageNode &s, long long step, int b, int64_t i,
+                                             int64_t idx, float I, float gam, float *g_out) {
+    const float k = (-s.Uv + I) + gam;
+    const float dt = (float)a.dt;
+    float Un;
+    if (a.stage == 1) {
+        a.ks[idx] = k;
+        Un = fmaf(0.5f * dt, k, s.uv);
+    } else if (a.stage == 2) {
+        a.ks[idx] = fmaf(2.f, k, s.ksv);
+        Un = fmaf(0.5f * dt, k, s.uv);
+    } else if (a.stage == 3) {
+        a.ks[idx] = fmaf(2.f, k, s.ksv);
+        Un = fmaf(dt, k, s.uv);
+    } else {
+        const float unew = fmaf(dt / 6.f, s.ksv + k, s.uv);
+        a.us[idx] = unew;
+        const int64_t cidx = (int64_t)b * a.n + s.node;
+        if (a.perm && a.u) a.u[cidx] = unew;
+        Un = unew;
+        if (!isfinite(unew) && *a.err == DEV_OK) atomicCAS(a.err, DEV_OK, DEV_NONFINITE);
+        if (a.ckpt && ((step + 1) % a.C) == 0) a.ckpt[(int64_t)((step + 1) / a.C) * a.B * a.n + cidx] = unew;
+    }
+    a.U[idx] = Un;
+    if (a.stage_out) a.stage_out[idx] = Un;
+    const float f = firing_rate(Un, s.bb, s.th);
+    g_out[(int64_t)b * a.n_pad + i] = a.q ? s.qv * f : f;
+}
+
+// End of a step (stage 4): the last of `blocks` blocks advances the device step counter.
+__device__ __forceinline__ void step_done(const StageKArgs &a, unsigned blocks) {
+    if (a.stage != 4) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned prev = atomicAdd(a.done_ctr, 1u);
+        if (prev == blocks - 1) {
+            *a.done_ctr = 0u;
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.step_ctr), 1ull);
+            __threadfence();
+        }
+    }
+}
+
+// ----------------------------------------------------------------------------
 // Single-trajectory variant on packed FP32 pairs (f32x2: one instruction, two lanes of
 // the FMA pipe).  Column tiles are staged as structure-of-arrays (x, y, z, g), so a
 // lane reads two adjacent columns with one 8-byte load; each row's coordinates are held
@@ -191,11 +359,25 @@ constexpr float kMfLocalSpread = 1.0f;
 
 // xyz: coordinates in exponent units as structure of arrays [x(n_pad) | y(n_pad) | z(n_pad)];
 // g_all: B x n_pad firing rates (times q); both in Hilbert order, like the partial sums.
-template <int R, int TJ, int M>
+//
+// MODE 0 writes partial sums.  Small node sets (MODE 1, 2: one column split, so a warp holds the
+// whole sums of its rows) finish in the same launch: MODE 1 performs the RK4 stage of its rows,
+// MODE 2 writes them to the caller's I.  At 1,500 nodes a sum is 1 us of arithmetic; what
+// counts is launches and their dependent loads, so the static tiles are staged before
+// pdl_wait(), the rows' state is read while the tiles are swept, and g alternates between two
+// buffers (other blocks still read this stage's while the first rows of the next are written).
+struct FusedOut {
+    StageKArgs st;  // MODE 1
+    float *g_next;  // MODE 1: the other g buffer
+    float *I;       // MODE 2, caller's order
+    const int *perm;
+    int64_t n;
+};
+template <int R, int TJ, int M, int MODE>
 __global__ void __launch_bounds__(MF_THREADS, R >= 8 ? 2 : 4)
 mf_pair_packed_kernel(const float *__restrict__ xyz, const float *__restrict__ g_all, int64_t n_pad, int B, int b_base,
                       int64_t jchunk, float k2, float A1, float A2, float per, float *__restrict__ partial,
-                      int *__restrict__ err) {
+                      int *__restrict__ err, const __grid_constant__ FusedOut fo) {
     static_assert(M >= 0 && M <= 4, "form M: 0 general, 1 one Gaussian, 2-4 width ratio");
     __shared__ __align__(128) MfPackedSmem<TJ> sm;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -214,18 +396,33 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *__restrict__ g
         mbar_fence_init();
     }
     __syncthreads();
-    auto issue = [&](int t) {
+    auto issue_xyz = [&](int t) {
         const int buf = t & 1;
         const int64_t jt = j0 + (int64_t)t * TJ;
         mbar_arrive_expect_tx(&sm.bar[buf], kTileBytes);
         bulk_g2s(sm.xs[buf], X + jt, TJ * 4, &sm.bar[buf]);
         bulk_g2s(sm.ys[buf], Y + jt, TJ * 4, &sm.bar[buf]);
         bulk_g2s(sm.zs[buf], Z + jt, TJ * 4, &sm.bar[buf]);
-        bulk_g2s(sm.gs[buf], g + jt, TJ * 4, &sm.bar[buf]);
     };
+    auto issue_g = [&](int t) { bulk_g2s(sm.gs[t & 1], g + j0 + (int64_t)t * TJ, TJ * 4, &sm.bar[t & 1]); };
     if (tid == 0) {
-        if (ntiles > 0) issue(0);
-        if (ntiles > 1) issue(1);
+        if (ntiles > 0) issue_xyz(0);
+        if (ntiles > 1) issue_xyz(1);
+    }
+    // MODE 1: lane r < R carries row r's state
+    long long step = 0;
+    StageNode sn{};
+    const int64_t own = slot0 + lane;
+    const bool mine = MODE != 0 && lane < R && own < fo.n;
+    pdl_wait();  // the kernel before wrote g and the rows' state
+    pdl_trigger();
+    if constexpr (MODE == 1) {
+        step = *fo.st.step_ctr;
+        if (mine) sn = stage_load(fo.st, b, own, (int64_t)b * fo.n + own);
+    }
+    if (tid == 0) {
+        if (ntiles > 0) issue_g(0);
+        if (ntiles > 1) issue_g(1);
     }
     // the warp's rows (all lanes hold the same values) and the centre of their bounding box
     float xr[R], yr[R], zr[R];
@@ -277,7 +474,10 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *__restrict__ g
             timed_out = true;
             break;
         }
-        if (tid == 0 && t >= 1 && t + 1 < ntiles) issue(t + 1);
+        if (tid == 0 && t >= 1 && t + 1 < ntiles) {
+            issue_xyz(t + 1);
+            issue_g(t + 1);
+        }
         const u64 *xs = reinterpret_cast<const u64 *>(sm.xs[buf]);
         const u64 *ys = reinterpret_cast<const u64 *>(sm.ys[buf]);
         const u64 *zs = reinterpret_cast<const u64 *>(sm.zs[buf]);
@@ -342,6 +542,7 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *__restrict__ g
         }
         return;
     }
+    float total = 0.f;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         float p0, p1, q0, q1;
@@ -357,8 +558,18 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *__restrict__ g
             s1f *= exp2f(M >= 2 ? -(float)M * ni : -ni);
             s2f *= exp2f(M >= 2 ? -ni : -k2 * ni);
         }
-        float v = warp_sum(s1f - s2f);
-        if (lane == 0) partial[((int64_t)split * B + b) * n_pad + slot0 + r] = v;
+        const float v = warp_sum(s1f - s2f);
+        if constexpr (MODE == 0) {
+            if (lane == 0) partial[((int64_t)split * B + b) * n_pad + slot0 + r] = v;
+        } else {
+            if (lane == r) total = v;
+        }
+    }
+    if constexpr (MODE == 1) {
+        if (mine) stage_update(fo.st, sn, step, b, own, (int64_t)b * fo.n + own, total, 0.f, fo.g_next);
+        step_done(fo.st, gridDim.x * gridDim.z);
+    } else if constexpr (MODE == 2) {
+        if (mine) fo.I[(int64_t)b * fo.n + fo.perm[own]] = total;
     }
 }
 
@@ -463,8 +674,8 @@ constexpr MfVariant kMfVariants[] = {{2, 512}, {4, 512}, {4, 1024}, {8, 1024}};
 template <int R, int TJ>
 static int packed_resident() {
     int nb0 = 0, nb4 = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb0, mf_pair_packed_kernel<R, TJ, 0>, MF_THREADS, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb4, mf_pair_packed_kernel<R, TJ, 4>, MF_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb0, mf_pair_packed_kernel<R, TJ, 0, 0>, MF_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb4, mf_pair_packed_kernel<R, TJ, 4, 0>, MF_THREADS, 0);
     return std::max(std::min(nb0, nb4), 1);
 }
 
@@ -483,13 +694,13 @@ static void launch_packed(nf_operator *op, int B, int b_base, int groups, const 
     const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
     dim3 grid((unsigned)pl.row_blocks, (unsigned)pl.splits, (unsigned)groups);
 #define NF_PACKED_ARGS \
-    op->xyz, op->g, op->n_pad, B, b_base, pl.jchunk, k2, k.A1, k.A2, mf_period(op), op->partial, op->err
+    op->xyz, op->g, op->n_pad, B, b_base, pl.jchunk, k2, k.A1, k.A2, mf_period(op), op->partial, op->err, FusedOut{}
     switch (op->form) {
-        case 1: mf_pair_packed_kernel<R, TJ, 1><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
-        case 2: mf_pair_packed_kernel<R, TJ, 2><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
-        case 3: mf_pair_packed_kernel<R, TJ, 3><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
-        case 4: mf_pair_packed_kernel<R, TJ, 4><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
-        default: mf_pair_packed_kernel<R, TJ, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
+        case 1: mf_pair_packed_kernel<R, TJ, 1, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
+        case 2: mf_pair_packed_kernel<R, TJ, 2, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
+        case 3: mf_pair_packed_kernel<R, TJ, 3, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
+        case 4: mf_pair_packed_kernel<R, TJ, 4, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
+        default: mf_pair_packed_kernel<R, TJ, 0, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
     }
 #undef NF_PACKED_ARGS
 }
@@ -506,6 +717,46 @@ static nf_status launch_mf_packed(nf_operator *op, int B, int b_base, int groups
     return NF_OK;
 }
 
+// Up to kSymMaxB trajectories take the symmetric kernel, one launch with a grid z per
+// trajectory: each trajectory's pairs are evaluated once, which beats the multi-trajectory
+// kernels (ordered pairs, exponentials shared across trajectories) until about four
+// trajectories (measured at n = 1e5: B = 2 in 4.9 ms and B = 3 in 7.7 ms there, against
+// 1.8 ms per symmetric trajectory; B = 4 in 5.4 ms).
+constexpr int kSymMaxB = 3;
+
+// Small node sets on the automatic schedule take one launch per sum: 2 rows per warp, columns in
+// tiles of 1,024 (one or two at most sizes here; 512-node tiles, 1 or 4 rows per warp measured
+// slower at most sizes).  Per RK4 stage on GB300, against the packed pair kernel and the stage
+// kernel with and without overlapped launches: n = 1,000 4.3 us (4.8, 5.9), 2,000 5.9 (6.4, 8.4),
+// 3,000 9.5 (9.4, 11.0); at 4,000 nodes 11.5, where the symmetric kernel on 256-node blocks takes
+// 9.5 (15.1 before), hence the line.
+constexpr int64_t kFusedMaxN = 3072;
+constexpr int kFusedRows = 2, kFusedTile = 1024;
+bool fused_fits(const nf_operator *op, int B) {
+    return op->path == NF_MATRIX_FREE && op->mf_sched == NF_MF_AUTO && !op->mf_cull && op->n <= kFusedMaxN &&
+           B <= kSymMaxB;
+}
+
+template <int MODE>
+static cudaError_t launch_fused(nf_operator *op, int B, const float *g, const FusedOut &fo, bool overlap, cudaStream_t s) {
+    constexpr int R = kFusedRows, TJ = kFusedTile;
+    const nf_kernel &k = op->kp;
+    const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
+    // row blocks with a real node only; every column tile
+    const dim3 grid((unsigned)ceil_div(op->n, MF_WARPS * R), 1, (unsigned)B);
+    auto go = [&](auto kernel) {
+        return launch_dependent(kernel, grid, MF_THREADS, 0, s, overlap, op->xyz, g, op->n_pad, B, 0, op->n_pad, k2,
+                                k.A1, k.A2, mf_period(op), (float *)nullptr, op->err, fo);
+    };
+    switch (op->form) {
+        case 1: return go(mf_pair_packed_kernel<R, TJ, 1, MODE>);
+        case 2: return go(mf_pair_packed_kernel<R, TJ, 2, MODE>);
+        case 3: return go(mf_pair_packed_kernel<R, TJ, 3, MODE>);
+        case 4: return go(mf_pair_packed_kernel<R, TJ, 4, MODE>);
+        default: return go(mf_pair_packed_kernel<R, TJ, 0, MODE>);
+    }
+}
+
 // Launch shape of the packed kernel (single trajectories inside a multi-trajectory call):
 // small node sets want more, smaller blocks.
 static int default_variant(int64_t n_pad) { return n_pad >= 16384 ? 3 : 0; }
@@ -517,20 +768,14 @@ static int64_t sym_pairs_1024(const nf_operator *op) {
 }
 int sym_slots(const nf_operator *op) { return (int)(op->n_pad / op->sym_blk); }
 
-// Up to kSymMaxB trajectories take the symmetric kernel, one launch with a grid z per
-// trajectory: each trajectory's pairs are evaluated once, which beats the multi-trajectory
-// kernels (ordered pairs, exponentials shared across trajectories) until about four
-// trajectories (measured at n = 1e5: B = 2 in 4.9 ms and B = 3 in 7.7 ms there, against
-// 1.8 ms per symmetric trajectory; B = 4 in 5.4 ms).
-constexpr int kSymMaxB = 3;
-
-// One trajectory takes the symmetric kernel when it has at least 2/3 as many block pairs as
-// the GPU has SMs; smaller node sets (below ~13,300 nodes on 152 SMs) have too few block
-// pairs to fill the GPU and take the packed row-block x column-split kernel instead, which
-// evaluates ordered pairs but spreads them over many more CTAs (measured crossover on GB300:
-// packed 0.119 ms vs symmetric 0.130 ms at n = 12,000; 0.155 vs 0.131 ms at n = 16,384).
+// Up to kSymMaxB trajectories take the symmetric kernel beyond kFusedMaxN nodes, on blocks of
+//   256 nodes  while 1,024-node block pairs are fewer than 2/3 of the SMs (n below ~13,300): the
+//              packed row-block x column-split kernel that served these sizes before evaluates
+//              ordered pairs (per RK4 stage, packed before / 256 / 512: n = 5,500 23.9 / 13.1 /
+//              20.8 us, 8,000 40.4 / 20.6 / 20.8, 13,000 82 / 41 / 43);
+//   512, 1,024 above, by timing (mf_autotune).
 // The automatic schedule also keeps the symmetric partial sums (one slot of n_pad floats per
-// 1,024-node block, growing as n^2) within an eighth of the device memory: beyond that (n
+// node block, growing as n^2) within an eighth of the device memory: beyond that (n
 // above about 3 million on a GB300) the packed kernel, whose layout grows with its column
 // splits only, takes over.
 static bool sym_layout_fits(const nf_operator *op) {
@@ -548,7 +793,7 @@ static bool sym_layout_fits(const nf_operator *op) {
 static bool use_sym(const nf_operator *op) {
     if (op->mf_sched == NF_MF_SYMMETRIC) return true;
     if (op->mf_sched == NF_MF_PACKED) return false;
-    return 3 * sym_pairs_1024(op) >= 2 * (int64_t)num_sms() && sym_layout_fits(op);
+    return op->n > kFusedMaxN && sym_layout_fits(op);
 }
 
 int mf_splits(nf_operator *op, int B) {
@@ -566,6 +811,12 @@ SplitPlan mf_plan(nf_operator *op) {
 
 // Shape of the single-trajectory (symmetric) launch: rows per warp, block width, slots.
 void mf_launch_shape(nf_operator *op, int *R, int *TJ, int *splits) {
+    if (fused_fits(op, 1)) {
+        *R = kFusedRows;
+        *TJ = kFusedTile;
+        *splits = 1;
+        return;
+    }
     if (!use_sym(op)) {
         const SplitPlan pl = mf_plan(op);
         *R = kMfVariants[op->mf_variant].R;
@@ -588,8 +839,11 @@ nf_status mf_autotune(nf_operator *op, cudaStream_t s) {
     static std::mutex mu;
     static std::map<std::tuple<int, int64_t, int>, int> cache;
     op->mf_variant = default_variant(op->n_pad);
-    if (3 * sym_pairs_1024(op) < 2 * (int64_t)num_sms() || !sym_layout_fits(op))
-        return NF_OK;  // packed by default
+    if (!sym_layout_fits(op)) return NF_OK;  // packed by default
+    if (3 * sym_pairs_1024(op) < 2 * (int64_t)num_sms()) {
+        op->sym_blk = op->n > kFusedMaxN ? 256 : 128;  // 128: only when the schedule asks for symmetric
+        return NF_OK;
+    }
     // 512-node blocks only where 1,024-node pairs fill fewer than four waves of two CTAs per
     // SM (n below ~49,000): four times the CTAs even out the last wave there
     if (sym_pairs_1024(op) >= 8 * (int64_t)num_sms()) return NF_OK;
@@ -850,17 +1104,14 @@ nf_status launch_mf_pair_single(const float4 *x4, const float *g, int64_t n_pad,
 // ----------------------------------------------------------------------------
 // Elementwise kernels.
 
-__device__ __forceinline__ float firing_rate(float u, float beta, float theta) {
-    return 1.0f / (1.0f + expf(-beta * (u - theta)));
-}
-
 // The elementwise kernels run over the operator's positions (thread idx = b n + p) and touch
 // the caller's arrays at node perm[p] (perm == nullptr: the same order).
 
-// g[b, p] = q_p f_b(u[b, perm[p]]) (q == nullptr: f alone);  optionally U[b, p] = u.
+// g[b, p] = q_p f_b(u[b, perm[p]]) (q == nullptr: f alone);  optionally U[b, p] = us[b, p] = u.
 __global__ void prep_g_kernel(const float *__restrict__ u, const int *__restrict__ perm, int64_t n, int64_t n_pad,
                               int B, const float *__restrict__ q, const float *__restrict__ beta,
-                              const float *__restrict__ theta, float *__restrict__ g, float *__restrict__ U) {
+                              const float *__restrict__ theta, float *__restrict__ g, float *__restrict__ U,
+                              float *__restrict__ us) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)B * n) return;
     const int b = (int)(idx / n);
@@ -869,6 +1120,7 @@ __global__ void prep_g_kernel(const float *__restrict__ u, const int *__restrict
     const float f = firing_rate(uv, beta[b], theta[b]);
     g[(int64_t)b * n_pad + j] = q ? q[j] * f : f;
     if (U) U[idx] = uv;
+    if (us) us[idx] = uv;
 }
 
 nf_status launch_prep_g(nf_operator *op, const float *u, int B, const float *beta, const float *theta,
@@ -877,7 +1129,8 @@ nf_status launch_prep_g(nf_operator *op, const float *u, int B, const float *bet
     const int T = 256;
     const bool mf = q_on_vector(op);
     prep_g_kernel<<<(unsigned)ceil_div(tot, T), T, 0, s>>>(u, op->perm, op->n, op->n_pad, B, mf ? op->q : nullptr,
-                                                          beta, theta, op->g, copy_to_U ? op->U : nullptr);
+                                                          beta, theta, op->g, copy_to_U ? op->U : nullptr,
+                                                          copy_to_U ? op->us : nullptr);
     NF_CUDA_TRY(cudaGetLastError());
     return NF_OK;
 }
@@ -885,6 +1138,7 @@ nf_status launch_prep_g(nf_operator *op, const float *u, int B, const float *bet
 __global__ void reduce_I_kernel(const float *__restrict__ partial, int splits, int64_t n, int64_t n_pad, int B,
                                 const float *__restrict__ rs, const int *__restrict__ perm, float *__restrict__ I) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (idx >= (int64_t)B * n) return;
     const int b = (int)(idx / n);
     const int64_t i = idx - (int64_t)b * n;
@@ -896,179 +1150,41 @@ nf_status launch_reduce_I(nf_operator *op, int B, int splits, float *I, cudaStre
     const int64_t tot = (int64_t)B * op->n;
     const int T = 256;
     const float *rs = (op->path == NF_DENSE_BF16X2) ? op->rs : nullptr;
-    reduce_I_kernel<<<(unsigned)ceil_div(tot, T), T, 0, s>>>(op->partial, splits, op->n, op->n_pad, B, rs, op->perm,
-                                                            I);
-    NF_CUDA_TRY(cudaGetLastError());
+    NF_CUDA_TRY(launch_dependent(reduce_I_kernel, dim3((unsigned)ceil_div(tot, T)), T, 0, s, true, op->partial, splits,
+                                 op->n, op->n_pad, B, rs, op->perm, I));
     return NF_OK;
 }
 
 // ----------------------------------------------------------------------------
-// Constants of the flat manufactured forcing (host side of forcing_value): per Gaussian of the
-// kernel with amplitude A and width w, p = 1 / w^2.
-struct FlatTerm {
-    double amp;        // +-A / (2 pi sigma^2)
-    double rs, prs;    // r / (p + r), -p r / (p + r)
-    double k;          // sqrt(p + r)
-    double half_root;  // sqrt(pi / (p + r)) / 2
-};
-struct FlatConst {
-    double L, iL, r, norm;  // period, 1 / (2 sigma^2), 1 / (2 pi sigma^2)
-    double c0;              // the convolution's constant part
-    FlatTerm t[2];
-    int terms;
-};
-
-// Fused RK4 stage: I = sum of splits; k_s = -U_s + I + gamma(t_s); RK4 bookkeeping;
-// next stage input and its g.  On the last stage the last block advances the
-// device step counter, so one captured step can be replayed.
-struct StageKArgs {
-    const float *partial;
-    int splits;
-    int64_t n, n_pad;
-    int B;
-    float *u, *U, *ks, *g;
-    const float *q;     // matrix-free: g = q f; dense: g = f (q lives in W)
-    const float *rs;    // BF16X2 row scale, or null
-    const float *beta, *theta;
-    nf_forcing F;
-    FlatConst fc;       // flat manufactured forcing
-    const float4 *x4;   // node coordinates (manufactured forcings)
-    const double *t0;
-    double dt;
-    int stage;
-    long long *step_ctr;
-    unsigned *done_ctr;
-    float *ckpt;
-    int C;
-    const int *perm;    // caller's node of each position (u, ckpt, Y1, Y2), or null
-    float *stage_out;   // next stage's input, kept by the adjoint's recomputation, or null
-    int *err;           // operator's device flag: DEV_NONFINITE on a non-finite new state
-};
-
-// Flat manufactured forcing (NF_FORCE_MMS_FLAT).  One factor of the convolution term:
-//   J(a) = int_{-L/2}^{L/2} exp(-p d^2) exp(-e(d)^2 / (2 sigma^2)) dd,  e(d) = nearest image of a - d,
-// a = nearest image of x - x0 in one coordinate.  e(d) = a - d except past the point where
-// a - d leaves [-L/2, L/2] (d < a - L/2 for a >= 0, d > a + L/2 for a < 0), where it is
-// a - d -+ L.  Each piece is a Gaussian product integrated in closed form:
-//   int_{d0}^{d1} exp(-p d^2 - r (d - a')^2) dd
-//     = exp(-p r a'^2 / (p + r)) (1/2) sqrt(pi / (p + r)) [erf(k (d1 - m)) - erf(k (d0 - m))],
-// r = 1 / (2 sigma^2), m = r a' / (p + r), k = sqrt(p + r).
-// The forcing is FP64 arithmetic on a chip whose FP64 pipe gives two lanes per clock per SM, so
-// what does not depend on the node is taken out: constants come from the host, cos t and sin t
-// from one thread per block, an erf is evaluated only where it is not +-1 to the last bit, and a
-// piece whose two erf agree is 0 without its exponential (all pieces but one, away from the
-// kink lines).
-constexpr double kPi = 3.14159265358979323846;
-__device__ __forceinline__ double erf_sat(double z) { return z >= 6.0 ? 1.0 : (z <= -6.0 ? -1.0 : erf(z)); }
-__device__ __forceinline__ double gauss_piece(const FlatTerm &g, double a, double d0, double d1) {
-    const double m = g.rs * a, diff = erf_sat(g.k * (d1 - m)) - erf_sat(g.k * (d0 - m));
-    return diff == 0.0 ? 0.0 : exp(g.prs * a * a) * g.half_root * diff;
-}
-__device__ __forceinline__ double flat_factor(const FlatTerm &g, double a, double L) {
-    const double h = 0.5 * L;
-    if (a >= 0.0) return gauss_piece(g, a - L, -h, a - h) + gauss_piece(g, a, a - h, h);
-    return gauss_piece(g, a, -h, a + h) + gauss_piece(g, a + L, a + h, h);
-}
-
-// i: position in the operator's order (x4); node: the caller's index (Y1, Y2); ct, sn = cos t, sin t
-__device__ __forceinline__ double forcing_value(const nf_forcing &F, const FlatConst &fc, const float4 *x4, int64_t i,
-                                                int64_t node, double ct, double sn, float beta, float theta) {
-    if (F.kind == NF_FORCE_MMS_FLAT) {
-        // z = G(x, x0(t); sigma) + c on the periodic square; gamma = du*/dt + u* - scale C,
-        // C = int_cell w(dist(x, y)) z(y) dy: the constant part integrates w over the
-        // displacement square, the Gaussian part is separable (flat_factor per coordinate)
-        const double x0 = F.radius * ct, y0 = F.radius * sn;
-        const float4 xi = x4[i];
-        double ax = (double)xi.x - x0, ay = (double)xi.y - y0;
-        ax -= fc.L * rint(ax * fc.iL);
-        ay -= fc.L * rint(ay * fc.iL);
-        const double G = exp(-(ax * ax + ay * ay) * fc.r) * fc.norm;
-        const double z = G + F.c;
-        const double dz = G * (ay * x0 - ax * y0) * (2.0 * fc.r);
-        const double us = (double)theta + log(z / (1.0 - z)) / (double)beta;
-        const double dus = dz / ((double)beta * z * (1.0 - z));
-        double C = fc.c0;
-        for (int h = 0; h < fc.terms; ++h)
-            C += fc.t[h].amp * (flat_factor(fc.t[h], ax, fc.L) * flat_factor(fc.t[h], ay, fc.L));
-        return dus + us - F.scale * C;
-    }
-    double Y1, Y2;
-    if (F.kind == NF_FORCE_MMS_SPHERE) {  // Y1 = z / 2 (degree 1), Y2 = x y (degree 2) at the node
-        const float4 xi = x4[i];
-        Y1 = 0.5 * (double)xi.z;
-        Y2 = (double)xi.x * (double)xi.y;
-    } else {
-        Y1 = F.Y1[node];
-        Y2 = F.Y2[node];
-    }
-    const double Y = Y1 + Y2;
-    const double a = F.a0 * ct, da = -F.a0 * sn;
-    const double z = F.c + a * Y;
-    const double us = (double)theta + log(z / (1.0 - z)) / (double)beta;
-    const double dus = da * Y / ((double)beta * z * (1.0 - z));
-    return dus + us - (F.lam0 * F.c + a * (F.lam1 * Y1 + F.lam2 * Y2));
-}
-
 __global__ void rk4_stage_kernel(StageKArgs a) {
+    // What earlier stage kernels wrote is complete (pdl_trigger of the pair kernel in between), so
+    // the state is read while the pair kernel still runs; only the partial sums wait for it.
     const long long step = *a.step_ctr;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    __shared__ double time_cs[2];  // cos t, sin t of the stage
+    const bool in = idx < (int64_t)a.B * a.n;
+    const int b = in ? (int)(idx / a.n) : 0;
+    const int64_t i = in ? idx - (int64_t)b * a.n : 0;
+    const StageNode sn = stage_load(a, b, i, in ? idx : 0);
+    const float rsv = a.rs ? a.rs[i] : 1.f;
+    float gam = 0.f;
     if (a.F.kind != NF_FORCE_NONE) {
+        __shared__ double time_cs[2];  // cos t, sin t of the stage
         if (threadIdx.x == 0) {
             const double cs = (a.stage == 1) ? 0.0 : (a.stage == 4 ? 1.0 : 0.5);
             const double ts = *a.t0 + (double)step * a.dt + cs * a.dt;
             sincos(ts, &time_cs[1], &time_cs[0]);
         }
         __syncthreads();
+        if (in) gam = (float)forcing_value(a.F, a.fc, a.x4, i, sn.node, time_cs[0], time_cs[1], sn.bb, sn.th);
     }
-    if (idx < (int64_t)a.B * a.n) {
-        const int b = (int)(idx / a.n);
-        const int64_t i = idx - (int64_t)b * a.n;
+    pdl_wait();
+    pdl_trigger();
+    if (in) {
         float I = sum_slots(a.partial + (int64_t)b * a.n_pad + i, (int64_t)a.B * a.n_pad, a.splits);
-        if (a.rs) I *= a.rs[i];
-        const float bb = a.beta[b], th = a.theta[b];
-        const int64_t node = a.perm ? a.perm[i] : i, cidx = (int64_t)b * a.n + node;
-        const float gam = a.F.kind == NF_FORCE_NONE
-                              ? 0.f
-                              : (float)forcing_value(a.F, a.fc, a.x4, i, node, time_cs[0], time_cs[1], bb, th);
-        const float Uv = a.U[idx], uv = a.u[cidx];
-        const float k = (-Uv + I) + gam;
-        const float dt = (float)a.dt;
-        float Un;
-        if (a.stage == 1) {
-            a.ks[idx] = k;
-            Un = fmaf(0.5f * dt, k, uv);
-        } else if (a.stage == 2) {
-            a.ks[idx] = fmaf(2.f, k, a.ks[idx]);
-            Un = fmaf(0.5f * dt, k, uv);
-        } else if (a.stage == 3) {
-            a.ks[idx] = fmaf(2.f, k, a.ks[idx]);
-            Un = fmaf(dt, k, uv);
-        } else {
-            const float unew = fmaf(dt / 6.f, a.ks[idx] + k, uv);
-            a.u[cidx] = unew;
-            Un = unew;
-            if (!isfinite(unew) && *a.err == DEV_OK) atomicCAS(a.err, DEV_OK, DEV_NONFINITE);
-            if (a.ckpt && ((step + 1) % a.C) == 0)
-                a.ckpt[(int64_t)((step + 1) / a.C) * a.B * a.n + cidx] = unew;
-        }
-        a.U[idx] = Un;
-        if (a.stage_out) a.stage_out[idx] = Un;
-        const float f = firing_rate(Un, bb, th);
-        a.g[(int64_t)b * a.n_pad + i] = a.q ? a.q[i] * f : f;
+        if (a.rs) I *= rsv;
+        stage_update(a, sn, step, b, i, idx, I, gam, a.g);
     }
-    if (a.stage == 4) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            const unsigned prev = atomicAdd(a.done_ctr, 1u);
-            if (prev == gridDim.x - 1) {
-                *a.done_ctr = 0u;
-                atomicAdd(reinterpret_cast<unsigned long long *>(a.step_ctr), 1ull);
-                __threadfence();
-            }
-        }
-    }
+    step_done(a, gridDim.x);
 }
 
 // Start a new nf_rk4_advance call: clock t0 and step counter 0.
@@ -1101,7 +1217,7 @@ static FlatConst flat_const(const nf_forcing &F, const nf_kernel &kp) {
     return c;
 }
 
-nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s) {
+static StageKArgs stage_args(nf_operator *op, int B, const StageParams &p) {
     StageKArgs a{};
     a.partial = op->partial;
     a.splits = p.splits;
@@ -1109,6 +1225,7 @@ nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_
     a.n_pad = op->n_pad;
     a.B = B;
     a.u = p.u;
+    a.us = op->perm ? op->us : p.u;
     a.U = op->U;
     a.ks = op->ks;
     a.g = op->g;
@@ -1129,10 +1246,31 @@ nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_
     a.err = op->err;
     a.perm = op->perm;
     a.stage_out = p.stage_out;
+    return a;
+}
+
+nf_status launch_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s) {
+    const StageKArgs a = stage_args(op, B, p);
     const int64_t tot = (int64_t)B * op->n;
     const int T = 256;
-    rk4_stage_kernel<<<(unsigned)ceil_div(tot, T), T, 0, s>>>(a);
-    NF_CUDA_TRY(cudaGetLastError());
+    NF_CUDA_TRY(launch_dependent(rk4_stage_kernel, dim3((unsigned)ceil_div(tot, T)), T, 0, s, p.overlap, a));
+    return NF_OK;
+}
+
+nf_status fused_stage(nf_operator *op, int B, const StageParams &p, cudaStream_t s) {
+    const int64_t half = (int64_t)B * op->n_pad;
+    float *const g_in = op->g + ((p.stage - 1) & 1) * half;
+    const FusedOut fo{stage_args(op, B, p), op->g + (p.stage & 1) * half, nullptr, op->perm, op->n};
+    NF_CUDA_TRY(launch_fused<1>(op, B, g_in, fo, p.overlap, s));
+    return NF_OK;
+}
+
+nf_status fused_apply(nf_operator *op, int B, float *I, cudaStream_t s) {
+    FusedOut fo{};
+    fo.I = I;
+    fo.perm = op->perm;
+    fo.n = op->n;
+    NF_CUDA_TRY(launch_fused<2>(op, B, op->g, fo, true, s));
     return NF_OK;
 }
 

@@ -38,6 +38,7 @@ __device__ __forceinline__ float model_rate(const ModelArgs &m, float u, float b
 
 struct ModelState {
     float *u, *s;            // caller's state (s: depression only); the rest in the operator's order
+    float *us, *ss;          // the state in the operator's order (u, s themselves without perm)
     float *U, *S;            // current stage inputs
     float *ku, *ksd;         // RK4 slope accumulators (u, s)
     float *hu, *hs;          // AB5 history: 5 slots of B x n each (u, s)
@@ -52,9 +53,15 @@ struct ModelState {
     const int *perm;         // caller's node of each position (u, s), or null
 };
 
-// Index of the caller's u, s for position i of trajectory b.
-__device__ __forceinline__ int64_t caller_idx(const ModelState &st, int b, int64_t i, int64_t idx) {
-    return st.perm ? (int64_t)b * st.n + st.perm[i] : idx;
+// The new state: kept in the operator's order, and written to the caller's arrays.
+__device__ __forceinline__ void write_state(const ModelState &st, bool dep, int b, int64_t i, int64_t idx, float u,
+                                            float s) {
+    st.us[idx] = u;
+    if (dep) st.ss[idx] = s;
+    if (!st.perm) return;
+    const int64_t c = (int64_t)b * st.n + st.perm[i];
+    st.u[c] = u;
+    if (dep) st.s[c] = s;
 }
 
 __device__ __forceinline__ void write_g(const ModelState &st, const ModelArgs &m, int b, int64_t i, int64_t idx,
@@ -76,11 +83,12 @@ __global__ void model_prep_kernel(ModelState st, ModelArgs m) {
     if (idx >= (int64_t)st.B * st.n) return;
     const int b = (int)(idx / st.n);
     const int64_t i = idx - (int64_t)b * st.n;
-    const int64_t ci = caller_idx(st, b, i, idx);
+    const bool dep = m.kind == NF_MODEL_DEPRESSION;
+    const int64_t ci = st.perm ? (int64_t)b * st.n + st.perm[i] : idx;
     const float u = st.u[ci];
-    const float s = (m.kind == NF_MODEL_DEPRESSION) ? st.s[ci] : 1.f;
-    st.U[idx] = u;
-    if (m.kind == NF_MODEL_DEPRESSION) st.S[idx] = s;
+    const float s = dep ? st.s[ci] : 1.f;
+    st.U[idx] = st.us[idx] = u;
+    if (dep) st.S[idx] = st.ss[idx] = s;
     write_g(st, m, b, i, idx, u, s);
 }
 
@@ -101,8 +109,7 @@ __global__ void model_rk4_stage_kernel(ModelState st, ModelArgs m, int stage, fl
         if (dep) st.hs[h] = ks;
     }
     float Un, Sn = 1.f;
-    const int64_t ci = caller_idx(st, b, i, idx);
-    const float uv = st.u[ci], sv = dep ? st.s[ci] : 1.f;
+    const float uv = st.us[idx], sv = dep ? st.ss[idx] : 1.f;
     if (stage == 1) {
         st.ku[idx] = ku;
         Un = fmaf(0.5f * dt, ku, uv);
@@ -120,11 +127,8 @@ __global__ void model_rk4_stage_kernel(ModelState st, ModelArgs m, int stage, fl
         }
     } else {
         Un = fmaf(dt / 6.f, st.ku[idx] + ku, uv);
-        st.u[ci] = Un;
-        if (dep) {
-            Sn = fmaf(dt / 6.f, st.ksd[idx] + ks, sv);
-            st.s[ci] = Sn;
-        }
+        if (dep) Sn = fmaf(dt / 6.f, st.ksd[idx] + ks, sv);
+        write_state(st, dep, b, i, idx, Un, Sn);
     }
     st.U[idx] = Un;
     if (dep) st.S[idx] = Sn;
@@ -140,8 +144,7 @@ __global__ void model_ab5_kernel(ModelState st, ModelArgs m, int step, float dt)
     const int64_t i = idx - (int64_t)b * st.n;
     const bool dep = m.kind == NF_MODEL_DEPRESSION;
     const int64_t plane = (int64_t)st.B * st.n;
-    const int64_t ci = caller_idx(st, b, i, idx);
-    const float uv = st.u[ci], sv = dep ? st.s[ci] : 1.f;
+    const float uv = st.us[idx], sv = dep ? st.ss[idx] : 1.f;
     const float Fu = -uv + slot_sum(st, b, i);
     const float Fs = dep ? (1.f - sv - m.beta_d * sv * model_rate(m, uv, st.beta[b], st.theta[b])) * m.tau_inv : 0.f;
     st.hu[(int64_t)(step % 5) * plane + idx] = Fu;
@@ -154,13 +157,8 @@ __global__ void model_ab5_kernel(ModelState st, ModelArgs m, int step, float dt)
         du = fmaf(c[k], st.hu[h], du);
         if (dep) ds = fmaf(c[k], st.hs[h], ds);
     }
-    const float un = fmaf(dt, du, uv);
-    st.u[ci] = un;
-    float sn = 1.f;
-    if (dep) {
-        sn = fmaf(dt, ds, sv);
-        st.s[ci] = sn;
-    }
+    const float un = fmaf(dt, du, uv), sn = dep ? fmaf(dt, ds, sv) : 1.f;
+    write_state(st, dep, b, i, idx, un, sn);
     write_g(st, m, b, i, idx, un, sn);
 }
 
@@ -186,18 +184,21 @@ extern "C" nf_status nf_field_advance(nf_operator *op, const nf_model *model, in
     const bool ab5 = integrator == NF_INTEGRATOR_AB5;
     const int64_t BN = (int64_t)B * op->n;
     NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B)));
-    float *extra = nullptr;  // S, ksd (depression), AB5 history u (and s)
-    const int64_t nextra = (dep ? 2 : 0) * BN + (ab5 ? (dep ? 10 : 5) * BN : 0);
+    float *extra = nullptr;  // S, ksd and, with perm, ss (depression), AB5 history u (and s)
+    const int64_t nextra = (dep ? (op->perm ? 3 : 2) : 0) * BN + (ab5 ? (dep ? 10 : 5) * BN : 0);
     if (nextra > 0) NF_CUDA_TRY(cudaMallocAsync(&extra, sizeof(float) * nextra, cs));
     ModelState st{};
     st.u = u;
     st.s = dep ? s : nullptr;
+    st.us = op->perm ? op->us : u;
     st.U = op->U;
     st.ku = op->ks;
     float *p = extra;
     if (dep) {
         st.S = p, p += BN;
         st.ksd = p, p += BN;
+        st.ss = st.s;
+        if (op->perm) st.ss = p, p += BN;
     }
     if (ab5) {
         st.hu = p, p += 5 * BN;

@@ -170,7 +170,7 @@ __global__ void query_kernel(const double *__restrict__ nodes, int dim, const in
 // other in `sorted`: FP32 offsets reject most nodes (with a margin for their rounding), the rest
 // get the exact FP64 distance and, if inside the radius, are ranked against each other by
 // (distance^2, index), each lane counting the entries before its own.  Against one thread per
-// query with its sorted list in local memory: 13 -> KNN_AFTER ms for 200,000 queries of k = 48.
+// query with its sorted list in local memory: 13 -> 2 ms for 200,000 queries of k = 48.
 // Queries whose radius holds more than KNN_CAP nodes, or too few comparable ones, are left to
 // knn_query_kernel (their row's first entry is -1).
 constexpr int KNN_CAP = 512, KNN_WARPS = 4;

@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(MS_THREADS, 2)
 mf_sym_kernel(SymNodes nd, const float *__restrict__ g_all, int B, int b_base, float k2, float per, float lim_tail,
               float lim_skip, float *__restrict__ partial, const int *__restrict__ pairs) {
     static_assert(M >= 0 && M <= 4, "form M: 0 general, 1 one Gaussian (A2 = 0), 2-4 width ratio");
-    static_assert(BLK == 512 || BLK == 1024, "block size");
+    static_assert(BLK >= 128 && BLK <= 1024 && (BLK & (BLK - 1)) == 0, "block size");
     constexpr int R = kPassRows, NPASS = BLK / R, NT = BLK / kTileCols;
     static_assert(NT <= 32 && NT * NT <= MS_THREADS, "one lane per tile, one thread per tile pair");
     // Integer width ratios combine the two Gaussians per pair: with the row factors f1, f2,
@@ -433,18 +433,37 @@ mf_sym_kernel(SymNodes nd, const float *__restrict__ g_all, int B, int b_base, f
         cp_async16(tcs + tid, nd.tc + cbase / kTileCols + tid);
         cp_async16(tes + tid, nd.te + cbase / kTileCols + tid);
     }
-    float gr[BLK / MS_THREADS];
-    bool bad = false, live = false;
+    constexpr int KT = (BLK + MS_THREADS - 1) / MS_THREADS;  // nodes per thread
+    float4 p[KT];
+    float2 w[KT];
 #pragma unroll
-    for (int t = 0; t < BLK / MS_THREADS; ++t) {
-        const float gc = __ldg(g + cbase + tid + t * MS_THREADS);
-        gr[t] = __ldg(g + rbase + tid + t * MS_THREADS);
-        gs[tid + t * MS_THREADS] = gc;
-        bad |= !(0.f * gc + 0.f * gr[t] == 0.f);  // 0 * v is NaN for a non-finite v
+    for (int t = 0; t < KT; ++t) {
+        const int k = min(tid + t * MS_THREADS, BLK - 1);
+        p[t] = __ldg(nd.rg + rbase + k);
+        w[t] = __ldg(nd.rw + rbase + k);
     }
+    bool bad = false, live = false;
     if (tid < NT * NT) {
         const int64_t ti = rbase / kTileCols + tid / NT, tj = cbase / kTileCols + tid % NT;
         live = box_d2(__ldg(nd.tc + ti), __ldg(nd.te + ti), __ldg(nd.tc + tj), __ldg(nd.te + tj), per, iper) <= lim_skip;
+    }
+    if (!diag)
+        for (int k = tid; k < MS_WARPS * BLK / 4; k += MS_THREADS)
+            reinterpret_cast<float4 *>(colacc)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // everything above depends on the operator alone; g is written by the kernel before
+    pdl_wait();
+    pdl_trigger();
+#pragma unroll
+    for (int t = 0; t < KT; ++t) {
+        const int k = tid + t * MS_THREADS;
+        if (k < BLK) {
+            const float gc = __ldg(g + cbase + k), gr = __ldg(g + rbase + k);
+            gs[k] = gc;
+            rg[k] = make_float4(p[t].x, p[t].y, p[t].z, CW ? w[t].x : w[t].x * gr);
+            rw[k] = w[t];
+            rh[k] = w[t].y * gr;
+            bad |= !(0.f * gc + 0.f * gr == 0.f);  // 0 * v is NaN for a non-finite v
+        }
     }
     if (!__syncthreads_or(bad || live)) {
         const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -456,18 +475,6 @@ mf_sym_kernel(SymNodes nd, const float *__restrict__ g_all, int B, int b_base, f
         return;
     }
     if (__syncthreads_or(bad)) lim_tail = lim_skip = __int_as_float(0x7f800000);
-#pragma unroll
-    for (int t = 0; t < BLK / MS_THREADS; ++t) {
-        const int k = tid + t * MS_THREADS;
-        const float4 p = __ldg(nd.rg + rbase + k);
-        const float2 w = __ldg(nd.rw + rbase + k);
-        rg[k] = make_float4(p.x, p.y, p.z, CW ? w.x : w.x * gr[t]);
-        rw[k] = w;
-        rh[k] = w.y * gr[t];
-    }
-    if (!diag)
-        for (int k = tid; k < MS_WARPS * BLK / 4; k += MS_THREADS)
-            reinterpret_cast<float4 *>(colacc)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     cp_async_wait_all();
     __syncthreads();
 
@@ -686,6 +693,9 @@ static cudaError_t sym_attrs() {
     cudaError_t e = sym_attr<M, 1024, false>();
     if (e == cudaSuccess) e = sym_attr<M, 1024, true>();
     if (e == cudaSuccess) e = sym_attr<M, 512, false>();
+    if (e == cudaSuccess) e = sym_attr<M, 512, true>();
+    if (e == cudaSuccess) e = sym_attr<M, 256, false>();
+    if (e == cudaSuccess) e = sym_attr<M, 128, false>();
     return e;
 }
 nf_status sym_init_attrs() {
@@ -698,7 +708,7 @@ nf_status sym_init_attrs() {
 }
 
 template <int BLK, bool D2>
-static void launch_sym_blk(nf_operator *op, int B, int b_base, cudaStream_t s) {
+static cudaError_t launch_sym_blk(nf_operator *op, int B, int b_base, cudaStream_t s) {
     const nf_kernel &k = op->kp;
     const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
     const int64_t nb = op->n_pad / BLK;
@@ -710,25 +720,37 @@ static void launch_sym_blk(nf_operator *op, int B, int b_base, cudaStream_t s) {
     const float per = mf_period(op);
     float tail, skip;
     class_limits(op, &tail, &skip);
-#define NF_SYM_ARGS nd, op->g, B, b_base, k2, per, tail, skip, op->partial, pairs
+    const float *g = op->g;
+    float *partial = op->partial;
+    auto go = [&](auto kernel) {
+        return launch_dependent(kernel, grid, MS_THREADS, smem, s, !op->profile, nd, g, B, b_base, k2, per, tail, skip,
+                                partial, pairs);
+    };
     switch (op->form) {
-        case 1: mf_sym_kernel<1, BLK, D2><<<grid, MS_THREADS, smem, s>>>(NF_SYM_ARGS); break;
-        case 2: mf_sym_kernel<2, BLK, D2><<<grid, MS_THREADS, smem, s>>>(NF_SYM_ARGS); break;
-        case 3: mf_sym_kernel<3, BLK, D2><<<grid, MS_THREADS, smem, s>>>(NF_SYM_ARGS); break;
-        case 4: mf_sym_kernel<4, BLK, D2><<<grid, MS_THREADS, smem, s>>>(NF_SYM_ARGS); break;
-        default: mf_sym_kernel<0, BLK, D2><<<grid, MS_THREADS, smem, s>>>(NF_SYM_ARGS); break;
+        case 1: return go(mf_sym_kernel<1, BLK, D2>);
+        case 2: return go(mf_sym_kernel<2, BLK, D2>);
+        case 3: return go(mf_sym_kernel<3, BLK, D2>);
+        case 4: return go(mf_sym_kernel<4, BLK, D2>);
+        default: return go(mf_sym_kernel<0, BLK, D2>);
     }
-#undef NF_SYM_ARGS
 }
 
 nf_status launch_sym(nf_operator *op, int B, int b_base, cudaStream_t s) {
-    if (op->sym_blk == 512)
-        launch_sym_blk<512, false>(op, B, b_base, s);
-    else if (op->planar)
-        launch_sym_blk<1024, true>(op, B, b_base, s);
-    else
-        launch_sym_blk<1024, false>(op, B, b_base, s);
-    NF_CUDA_TRY(cudaGetLastError());
+    switch (op->sym_blk) {
+        case 128: NF_CUDA_TRY((launch_sym_blk<128, false>(op, B, b_base, s))); break;
+        case 256: NF_CUDA_TRY((launch_sym_blk<256, false>(op, B, b_base, s))); break;
+        case 512:
+            if (op->planar)
+                NF_CUDA_TRY((launch_sym_blk<512, true>(op, B, b_base, s)));
+            else
+                NF_CUDA_TRY((launch_sym_blk<512, false>(op, B, b_base, s)));
+            break;
+        default:
+            if (op->planar)
+                NF_CUDA_TRY((launch_sym_blk<1024, true>(op, B, b_base, s)));
+            else
+                NF_CUDA_TRY((launch_sym_blk<1024, false>(op, B, b_base, s)));
+    }
     return NF_OK;
 }
 
