@@ -19,8 +19,9 @@
 //   NF_DENSE_SYM_BF16X2: the same blocks as bf16 hi + lo planes with symmetric power-of-two
 //                    scaling s_i s_j (the vector is scaled on the way in, each output by its
 //                    own s_i): the precision form of the symmetric operator.
-// Work items (32-row block, column split) write partial sums like the matrix-free
-// kernel, so the same stage kernel finishes the RK4 step.
+// Several trajectories share one stream of the matrix (passes of up to 8 on the full planes, up to
+// 4 on the symmetric ones).  Work items (32-row block, column split) write partial sums like the
+// matrix-free kernel, so the same stage kernel finishes the RK4 step.
 #include "nf_pairs.cuh"
 
 #include <algorithm>
@@ -245,282 +246,246 @@ __device__ __forceinline__ uint4 ld_stream_u4(const void *p) {
     return v;
 }
 
-// FP32 plane.  Lane l of a warp covers columns tile + 4l + 128u, u = 0..7.
-__global__ void __launch_bounds__(DG_THREADS)
-gemv_fp32_kernel(const float *__restrict__ W, const float *__restrict__ F, int64_t n_pad, int B, int b,
-                 int64_t jchunk, float *__restrict__ partial) {
+// Sums of NB trajectories over the full plane: W is streamed once for all of them (it was once per
+// trajectory).  A warp takes 4 rows; every W value it loads meets NB vector values from L1.  HL:
+// bf16 hi + lo planes in the blocked layout, lane l on columns tile + 8 l + 256 u; else the FP32
+// plane, columns tile + 4 l + 128 u.  Bound: HBM, 4 bytes per entry whatever NB: per RK4 stage at
+// n = 30,000 on the bf16 planes 1, 2, 3, 4, 8 trajectories in 525, 529, 526, 552, 644 us (559,
+// 1,112, 1,667, 2,219, 4,450 with one stream each).  Two CTAs per SM at 128 registers beat one
+// with more (3 trajectories 526 against 689 us).
+template <int NB, bool HL>
+__global__ void __launch_bounds__(DG_THREADS, NB == 1 && HL ? 4 : 2)
+gemv_kernel(const void *__restrict__ W0, const uint16_t *__restrict__ Wlo, const float *__restrict__ F, int64_t n_pad,
+            int B, int b0, int64_t jchunk, float *__restrict__ partial) {
+    constexpr int C = HL ? 8 : 4;                 // columns per load
+    constexpr int UB = (HL ? 2 : 4) / (NB > 4 ? 2 : 1);  // loads per row in flight: 16 (8) x 16 bytes a lane
+    constexpr int NU = DG_TILE / (32 * C);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int split = blockIdx.y;
     const int64_t row0 = ((int64_t)blockIdx.x * DG_WARPS + warp) * DG_R;
     const int64_t j0 = (int64_t)split * jchunk, j1 = min(n_pad, j0 + jchunk);
-    const float *Fb = F + (int64_t)b * n_pad;
-    float acc[DG_R] = {0.f, 0.f, 0.f, 0.f};
+    const float *Fb = F + (int64_t)b0 * n_pad;
+    const float *W32 = static_cast<const float *>(W0);
+    const uint16_t *Whi = static_cast<const uint16_t *>(W0);
+    float acc[DG_R][NB];
+#pragma unroll
+    for (int r = 0; r < DG_R; ++r)
+#pragma unroll
+        for (int v = 0; v < NB; ++v) acc[r][v] = 0.f;
+    pdl_wait();
+    pdl_trigger();
     for (int64_t t = j0; t < j1; t += DG_TILE) {
 #pragma unroll
-        for (int uh = 0; uh < 8; uh += 4) {
-            float4 w[DG_R][4];
+        for (int uh = 0; uh < NU; uh += UB) {
+            uint4 h[DG_R][UB], l[DG_R][HL ? UB : 1];
 #pragma unroll
             for (int r = 0; r < DG_R; ++r)
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    w[r][u] = ld_stream_f4(W + (row0 + r) * n_pad + t + 128 * (uh + u) + 4 * lane);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 f = __ldg(reinterpret_cast<const float4 *>(Fb + t + 128 * (uh + u) + 4 * lane));
-#pragma unroll
-                for (int r = 0; r < DG_R; ++r) {
-                    acc[r] = fmaf(w[r][u].x, f.x, acc[r]);
-                    acc[r] = fmaf(w[r][u].y, f.y, acc[r]);
-                    acc[r] = fmaf(w[r][u].z, f.z, acc[r]);
-                    acc[r] = fmaf(w[r][u].w, f.w, acc[r]);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < DG_R; ++r) {
-        const float v = warp_sum(acc[r]);
-        if (lane == 0) partial[((int64_t)split * B + b) * n_pad + row0 + r] = v;
-    }
-}
-
-// BF16 hi + lo planes.  Lane l covers columns tile + 8l + 256u, u = 0..3.
-__global__ void __launch_bounds__(DG_THREADS)
-gemv_bf16x2_kernel(const uint16_t *__restrict__ Whi, const uint16_t *__restrict__ Wlo, const float *__restrict__ F,
-                   int64_t n_pad, int B, int b, int64_t jchunk, float *__restrict__ partial) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int split = blockIdx.y;
-    const int64_t row0 = ((int64_t)blockIdx.x * DG_WARPS + warp) * DG_R;
-    const int64_t j0 = (int64_t)split * jchunk, j1 = min(n_pad, j0 + jchunk);
-    const float *Fb = F + (int64_t)b * n_pad;
-    float acc[DG_R] = {0.f, 0.f, 0.f, 0.f};
-    for (int64_t t = j0; t < j1; t += DG_TILE) {
-#pragma unroll
-        for (int uh = 0; uh < 4; uh += 2) {
-            uint4 h[DG_R][2], l[DG_R][2];
-#pragma unroll
-            for (int r = 0; r < DG_R; ++r)
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int64_t off = blocked_offset(row0 + r, t + 256 * (uh + u) + 8 * lane, n_pad);
-                    h[r][u] = ld_stream_u4(Whi + off);
-                    l[r][u] = ld_stream_u4(Wlo + off);
+                for (int u = 0; u < UB; ++u) {
+                    const int64_t col = t + 32 * C * (uh + u) + C * lane;
+                    if constexpr (HL) {
+                        const int64_t off = blocked_offset(row0 + r, col, n_pad);
+                        h[r][u] = ld_stream_u4(Whi + off);
+                        l[r][u] = ld_stream_u4(Wlo + off);
+                    } else {
+                        h[r][u] = ld_stream_u4(W32 + (row0 + r) * n_pad + col);
+                    }
                 }
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const float *fp = Fb + t + 256 * (uh + u) + 8 * lane;
-                const float4 f0 = __ldg(reinterpret_cast<const float4 *>(fp));
-                const float4 f1 = __ldg(reinterpret_cast<const float4 *>(fp + 4));
-                const float fv[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+            for (int u = 0; u < UB; ++u) {
+                const float *fp = Fb + t + 32 * C * (uh + u) + C * lane;
+                float fv[NB][C];
+#pragma unroll
+                for (int v = 0; v < NB; ++v)
+#pragma unroll
+                    for (int c = 0; c < C; c += 4) {
+                        const float4 f = __ldg(reinterpret_cast<const float4 *>(fp + (int64_t)v * n_pad + c));
+                        fv[v][c] = f.x, fv[v][c + 1] = f.y, fv[v][c + 2] = f.z, fv[v][c + 3] = f.w;
+                    }
 #pragma unroll
                 for (int r = 0; r < DG_R; ++r) {
+                    float w[C];
                     const uint32_t hw[4] = {h[r][u].x, h[r][u].y, h[r][u].z, h[r][u].w};
-                    const uint32_t lw[4] = {l[r][u].x, l[r][u].y, l[r][u].z, l[r][u].w};
+                    if constexpr (HL) {
+                        const uint32_t lw[4] = {l[r][u].x, l[r][u].y, l[r][u].z, l[r][u].w};
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float h0 = __uint_as_float(hw[q] << 16), h1 = __uint_as_float(hw[q] & 0xffff0000u);
-                        const float l0 = __uint_as_float(lw[q] << 16), l1 = __uint_as_float(lw[q] & 0xffff0000u);
-                        acc[r] = fmaf(h0 + l0, fv[2 * q], acc[r]);
-                        acc[r] = fmaf(h1 + l1, fv[2 * q + 1], acc[r]);
+                        for (int q = 0; q < 4; ++q) {
+                            w[2 * q] = __uint_as_float(hw[q] << 16) + __uint_as_float(lw[q] << 16);
+                            w[2 * q + 1] = __uint_as_float(hw[q] & 0xffff0000u) + __uint_as_float(lw[q] & 0xffff0000u);
+                        }
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) w[q] = __uint_as_float(hw[q]);
                     }
+#pragma unroll
+                    for (int v = 0; v < NB; ++v)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) acc[r][v] = fmaf(w[c], fv[v][c], acc[r][v]);
                 }
             }
         }
     }
 #pragma unroll
-    for (int r = 0; r < DG_R; ++r) {
-        const float v = warp_sum(acc[r]);
-        if (lane == 0) partial[((int64_t)split * B + b) * n_pad + row0 + r] = v;
-    }
+    for (int r = 0; r < DG_R; ++r)
+#pragma unroll
+        for (int v = 0; v < NB; ++v) {
+            const float s = warp_sum(acc[r][v]);
+            if (lane == 0) partial[((int64_t)split * B + b0 + v) * n_pad + row0 + r] = s;
+        }
 }
 
-// One CTA per stored block pair (I <= J).  Warp w takes rows w, w + 8, ... of the block;
-// lane l covers the columns 4 l + 128 u (u = 0..7) with 16-byte streaming loads.  Row sums:
-// dot products with g_J (shared memory), 8 rows at a time reduced across the warp by a
-// transposed butterfly; column sums: per lane in registers over the warp's 128 rows,
-// then added over the warps in a fixed order.  Diagonal blocks write their row sums only.
+// Symmetric blocks, up to NB trajectories per stream of the matrix.  A cluster of S CTAs takes one
+// stored block pair (I <= J), 1024 / S rows each (S > 1 where the pairs alone would leave most of
+// the GPU idle: 36 pairs at n = 8,000).  The columns are swept in NB parts of 1024 / NB, so that a
+// lane's share of the vectors and of the column sums stays in 32 registers each whatever NB:
+// warp w takes rows w, w + 8, ...; per row and part a lane loads 32 / NB columns with 16-byte
+// streaming loads; the row's dot products with g_J are reduced 8 rows at a time across the warp
+// by a transposed butterfly and added over the parts in shared memory; the column sums with
+// g_I are added over the warps, then over the cluster's CTAs through distributed shared memory,
+// each in a fixed order.  Row sums go to partial slot J, column sums to slot I; diagonal blocks
+// write their row sums only.
+//   HL: bf16 hi + lo blocks with symmetric scales: the vector is scaled on the way in
+// (g'_j = s_j g_j) and each output by its own s_i.
+template <int NB>
+constexpr size_t sym_smem_floats(int rows) {
+    return (size_t)2 * NB * rows + (size_t)SYM_WARPS * SB + (size_t)NB * SB;
+}
+template <int NB, bool HL>
 __global__ void __launch_bounds__(SYM_THREADS, 2)
-gemv_sym_fp32_kernel(const float *__restrict__ K, const float *__restrict__ g_all, int64_t n_pad, int B, int b,
-                     float *__restrict__ partial) {
-    __shared__ __align__(16) float gI[SB], gJ[SB];
-    __shared__ __align__(16) float colred[SYM_WARPS][SB];
+gemv_sym_kernel(const void *__restrict__ K, const float *__restrict__ g_all, const float *__restrict__ sc,
+                int64_t n_pad, int B, int b0, int rows, float *__restrict__ partial) {
+    constexpr int COLS = SB / NB;    // columns per part
+    constexpr int CL = 32 / NB;      // columns per lane and part
+    constexpr int RB = NB;           // rows in flight: 8 16-byte loads per lane
+    extern __shared__ __align__(16) float gs_smem[];
+    float *gI = gs_smem;                      // [NB][rows]
+    float *rowacc = gI + NB * rows;           // [NB][rows]
+    float *colred = rowacc + NB * rows;       // [SYM_WARPS][NB][COLS]
+    float *colsum = colred + SYM_WARPS * SB;  // [NB][SB]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     int I, J;
     sym_pair(blockIdx.x, I, J);
     const bool diag = I == J;
-    const float *g = g_all + (int64_t)b * n_pad;
-    for (int k = tid; k < SB; k += SYM_THREADS) {
-        gI[k] = g[(int64_t)I * SB + k];
-        gJ[k] = g[(int64_t)J * SB + k];
+    const int slice = blockIdx.y, row_off = slice * rows, nv = min(NB, B - b0);
+    // lane's column c of a part: FP32 4 lane + 128 u + (c & 3), u = c / 4; HL 8 lane + 256 u + (c & 7)
+    auto col_of = [&](int c) { return HL ? 8 * lane + 256 * (c >> 3) + (c & 7) : 4 * lane + 128 * (c >> 2) + (c & 3); };
+    pdl_wait();
+    pdl_trigger();
+    for (int k = tid; k < NB * rows; k += SYM_THREADS) {
+        const int v = k / rows, r = k - v * rows;
+        const int64_t node = (int64_t)I * SB + row_off + r;
+        float x = v < nv ? g_all[(int64_t)(b0 + v) * n_pad + node] : 0.f;
+        if constexpr (HL) x *= sc[node];
+        gI[k] = x;
     }
     __syncthreads();
-    const float *blk = K + (int64_t)blockIdx.x * SB * SB;
-    float col[32];
+    const float *blk32 = static_cast<const float *>(K) + (int64_t)blockIdx.x * SB * SB;
+    const uint4 *blkhl = static_cast<const uint4 *>(K) + (int64_t)blockIdx.x * SB * SBC * 2;
+    for (int part = 0; part < NB; ++part) {
+        float gj[NB][CL], col[NB][CL];
 #pragma unroll
-    for (int c = 0; c < 32; ++c) col[c] = 0.f;
-    float *out_rows = partial + ((int64_t)J * B + b) * n_pad + (int64_t)I * SB;
-    for (int r0 = warp; r0 < SB; r0 += 8 * SYM_WARPS) {  // 8 rows per group: r0, r0 + 8, ..., r0 + 56
-        float dot[8];
+        for (int c = 0; c < CL; c += 4) {
+            const int64_t node = (int64_t)J * SB + part * COLS + col_of(c);
+            float4 s4 = make_float4(1.f, 1.f, 1.f, 1.f);
+            if constexpr (HL) s4 = __ldg(reinterpret_cast<const float4 *>(sc + node));
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int r = r0 + 8 * k;
-            const float *row = blk + (int64_t)r * SB;
-            float4 v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = ld_stream_f4(row + 4 * lane + 128 * u);
-            const float gi = gI[r];
-            float d = 0.f;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float4 gj = *reinterpret_cast<const float4 *>(gJ + 4 * lane + 128 * u);
-                d = fmaf(v[u].x, gj.x, d);
-                d = fmaf(v[u].y, gj.y, d);
-                d = fmaf(v[u].z, gj.z, d);
-                d = fmaf(v[u].w, gj.w, d);
-                col[4 * u] = fmaf(v[u].x, gi, col[4 * u]);
-                col[4 * u + 1] = fmaf(v[u].y, gi, col[4 * u + 1]);
-                col[4 * u + 2] = fmaf(v[u].z, gi, col[4 * u + 2]);
-                col[4 * u + 3] = fmaf(v[u].w, gi, col[4 * u + 3]);
+            for (int v = 0; v < NB; ++v) {
+                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (v < nv) f = __ldg(reinterpret_cast<const float4 *>(g_all + (int64_t)(b0 + v) * n_pad + node));
+                gj[v][c] = f.x * s4.x, gj[v][c + 1] = f.y * s4.y, gj[v][c + 2] = f.z * s4.z, gj[v][c + 3] = f.w * s4.w;
+                col[v][c] = col[v][c + 1] = col[v][c + 2] = col[v][c + 3] = 0.f;
             }
-            dot[k] = d;
         }
-        // transposed butterfly: 7 shuffles reduce the 8 rows' dot products over the warp
-        int base = 0, cnt = 8;
+        for (int r0 = warp; r0 < rows; r0 += 8 * SYM_WARPS) {  // 8 rows per group: r0, r0 + 8, ..., r0 + 56
+            float dot[NB][8];
 #pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            if (cnt > 1) {
-                const int h = cnt >> 1;
-                const bool upper = (lane & off) != 0;
+            for (int kk = 0; kk < 8; kk += RB) {
+                float w[RB][CL];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (k < h) {
-                        const float send = upper ? dot[k] : dot[k + h];
-                        const float keep = upper ? dot[k + h] : dot[k];
-                        dot[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                for (int q = 0; q < RB; ++q) {
+                    const int64_t r = row_off + r0 + 8 * (kk + q);
+                    if constexpr (HL) {
+#pragma unroll
+                        for (int u = 0; u < CL / 8; ++u) {
+                            const uint4 *p = blkhl + (r * SBC + part * (COLS / 8) + lane + 32 * u) * 2;
+                            const uint4 hv = ld_stream_u4(p), lv = ld_stream_u4(p + 1);
+                            const uint32_t hw[4] = {hv.x, hv.y, hv.z, hv.w}, lw[4] = {lv.x, lv.y, lv.z, lv.w};
+#pragma unroll
+                            for (int t = 0; t < 4; ++t) {
+                                w[q][8 * u + 2 * t] = __uint_as_float(hw[t] << 16) + __uint_as_float(lw[t] << 16);
+                                w[q][8 * u + 2 * t + 1] =
+                                    __uint_as_float(hw[t] & 0xffff0000u) + __uint_as_float(lw[t] & 0xffff0000u);
+                            }
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < CL / 4; ++u) {
+                            const float4 f = ld_stream_f4(blk32 + r * SB + part * COLS + 4 * lane + 128 * u);
+                            w[q][4 * u] = f.x, w[q][4 * u + 1] = f.y, w[q][4 * u + 2] = f.z, w[q][4 * u + 3] = f.w;
+                        }
                     }
                 }
-                if (upper) base += h;
-                cnt = h;
-            } else {
-                dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], off);
-            }
-        }
-        if ((lane & 3) == 0) out_rows[r0 + 8 * base] = dot[0];
-    }
-    if (diag) return;
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-        *reinterpret_cast<float4 *>(&colred[warp][4 * lane + 128 * u]) =
-            make_float4(col[4 * u], col[4 * u + 1], col[4 * u + 2], col[4 * u + 3]);
-    __syncthreads();
-    float *out_cols = partial + ((int64_t)I * B + b) * n_pad + (int64_t)J * SB;
-    for (int k = tid; k < SB; k += SYM_THREADS) {
-        float v = 0.f;
+                for (int q = 0; q < RB; ++q)
 #pragma unroll
-        for (int w = 0; w < SYM_WARPS; ++w) v += colred[w][k];
-        out_cols[k] = v;
-    }
-}
-
-// Symmetric bf16 hi + lo blocks: gemv_sym_fp32_kernel's schedule on the scaled planes.  The
-// vector is scaled on the way into shared memory (g'_j = s_j g_j) and each output by its own
-// s_i, so one stored tile serves I_i = s_i sum_j (hi + lo)_ij g'_j (rows, slot J) and
-// I_j = s_j sum_i (hi + lo)_ij g'_i (columns, slot I).  Lane l reads chunks l + 32 u
-// (u = 0..3) of a row: 8 columns of hi and of lo, 32 contiguous bytes.
-__global__ void __launch_bounds__(SYM_THREADS, 2)
-gemv_sym_bf16x2_kernel(const uint4 *__restrict__ K, const float *__restrict__ g_all, const float *__restrict__ sc,
-                       int64_t n_pad, int B, int b, float *__restrict__ partial) {
-    __shared__ __align__(16) float gI[SB], gJ[SB];
-    __shared__ __align__(16) float colred[SYM_WARPS][SB];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int I, J;
-    sym_pair(blockIdx.x, I, J);
-    const bool diag = I == J;
-    const float *g = g_all + (int64_t)b * n_pad;
-    for (int k = tid; k < SB; k += SYM_THREADS) {
-        gI[k] = g[(int64_t)I * SB + k] * sc[(int64_t)I * SB + k];
-        gJ[k] = g[(int64_t)J * SB + k] * sc[(int64_t)J * SB + k];
-    }
-    __syncthreads();
-    const uint4 *blk = K + (int64_t)blockIdx.x * SB * SBC * 2;
-    float col[32];
+                    for (int v = 0; v < NB; ++v) {
+                        const float gi = gI[v * rows + r0 + 8 * (kk + q)];
+                        float d = 0.f;
 #pragma unroll
-    for (int c = 0; c < 32; ++c) col[c] = 0.f;
-    float *out_rows = partial + ((int64_t)J * B + b) * n_pad + (int64_t)I * SB;
-    for (int r0 = warp; r0 < SB; r0 += 8 * SYM_WARPS) {  // 8 rows per group: r0, r0 + 8, ..., r0 + 56
-        float dot[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int r = r0 + 8 * k;
-            const uint4 *row = blk + (int64_t)r * SBC * 2;
-            uint4 hv[4], lv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                hv[u] = ld_stream_u4(row + 2 * (lane + 32 * u));
-                lv[u] = ld_stream_u4(row + 2 * (lane + 32 * u) + 1);
-            }
-            const float gi = gI[r];
-            float d = 0.f;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 g0 = *reinterpret_cast<const float4 *>(gJ + 8 * (lane + 32 * u));
-                const float4 g1 = *reinterpret_cast<const float4 *>(gJ + 8 * (lane + 32 * u) + 4);
-                const float gj[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-                const uint32_t hw[4] = {hv[u].x, hv[u].y, hv[u].z, hv[u].w};
-                const uint32_t lw[4] = {lv[u].x, lv[u].y, lv[u].z, lv[u].w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float v0 = __uint_as_float(hw[q] << 16) + __uint_as_float(lw[q] << 16);
-                    const float v1 = __uint_as_float(hw[q] & 0xffff0000u) + __uint_as_float(lw[q] & 0xffff0000u);
-                    d = fmaf(v0, gj[2 * q], d);
-                    d = fmaf(v1, gj[2 * q + 1], d);
-                    col[8 * u + 2 * q] = fmaf(v0, gi, col[8 * u + 2 * q]);
-                    col[8 * u + 2 * q + 1] = fmaf(v1, gi, col[8 * u + 2 * q + 1]);
-                }
-            }
-            dot[k] = d;
-        }
-        int base = 0, cnt = 8;
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) {
-            if (cnt > 1) {
-                const int h = cnt >> 1;
-                const bool upper = (lane & off) != 0;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    if (k < h) {
-                        const float send = upper ? dot[k] : dot[k + h];
-                        const float keep = upper ? dot[k + h] : dot[k];
-                        dot[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                        for (int c = 0; c < CL; ++c) {
+                            d = fmaf(w[q][c], gj[v][c], d);
+                            col[v][c] = fmaf(w[q][c], gi, col[v][c]);
+                        }
+                        dot[v][kk + q] = d;
                     }
-                }
-                if (upper) base += h;
-                cnt = h;
-            } else {
-                dot[0] += __shfl_xor_sync(0xffffffffu, dot[0], off);
+            }
+#pragma unroll
+            for (int v = 0; v < NB; ++v) {
+                int row;
+                const float tot = warp_reduce_rows<8>(dot[v], lane, row);
+                float *dst = rowacc + v * rows + r0 + 8 * row;
+                if ((lane & 3) == 0) *dst = part == 0 ? tot : *dst + tot;
             }
         }
-        if ((lane & 3) == 0) {
-            const int r = r0 + 8 * base;
-            out_rows[r] = sc[(int64_t)I * SB + r] * dot[0];
+        if (!diag) {
+#pragma unroll
+            for (int v = 0; v < NB; ++v)
+#pragma unroll
+                for (int c = 0; c < CL; c += 4)
+                    *reinterpret_cast<float4 *>(colred + (warp * NB + v) * COLS + col_of(c)) =
+                        make_float4(col[v][c], col[v][c + 1], col[v][c + 2], col[v][c + 3]);
+            __syncthreads();
+            for (int k = tid; k < SB; k += SYM_THREADS) {
+                const int v = k / COLS, c = k - v * COLS;
+                float s = 0.f;
+#pragma unroll
+                for (int w = 0; w < SYM_WARPS; ++w) s += colred[(w * NB + v) * COLS + c];
+                colsum[v * SB + part * COLS + c] = s;
+            }
+            __syncthreads();
         }
     }
-    if (diag) return;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        float *dst = &colred[warp][8 * (lane + 32 * u)];
-        *reinterpret_cast<float4 *>(dst) = make_float4(col[8 * u], col[8 * u + 1], col[8 * u + 2], col[8 * u + 3]);
-        *reinterpret_cast<float4 *>(dst + 4) =
-            make_float4(col[8 * u + 4], col[8 * u + 5], col[8 * u + 6], col[8 * u + 7]);
-    }
     __syncthreads();
-    float *out_cols = partial + ((int64_t)I * B + b) * n_pad + (int64_t)J * SB;
-    for (int k = tid; k < SB; k += SYM_THREADS) {
-        float v = 0.f;
-#pragma unroll
-        for (int w = 0; w < SYM_WARPS; ++w) v += colred[w][k];
-        out_cols[k] = sc[(int64_t)J * SB + k] * v;
+    for (int k = tid; k < nv * rows; k += SYM_THREADS) {
+        const int v = k / rows, r = k - v * rows;
+        const int64_t node = (int64_t)I * SB + row_off + r;
+        partial[((int64_t)J * B + b0 + v) * n_pad + node] = HL ? sc[node] * rowacc[k] : rowacc[k];
     }
+    if (diag) return;  // uniform over the cluster
+    const int S = SB / rows;
+    if (S > 1) cluster_barrier();
+    for (int k = tid; k < nv * rows; k += SYM_THREADS) {  // this CTA's share of the columns
+        const int v = k / rows, c = row_off + (k - v * rows);
+        float s = 0.f;
+        if (S == 1) {
+            s = colsum[v * SB + c];
+        } else {
+            for (int q = 0; q < S; ++q) s += ld_cluster(colsum + v * SB + c, (uint32_t)q);
+        }
+        const int64_t node = (int64_t)J * SB + c;
+        partial[((int64_t)I * B + b0 + v) * n_pad + node] = HL ? sc[node] * s : s;
+    }
+    if (S > 1) cluster_barrier();  // no CTA leaves while another may read its sums
 }
 
 // ---------------------------------------------------------------- GEMM (several trajectories)
@@ -537,7 +502,8 @@ gemv_sym_bf16x2_kernel(const uint4 *__restrict__ K, const float *__restrict__ g_
 // memory (transposed: k-major).  Small node sets split K (grid z) into partial-sum slots
 // that the stage kernel adds in a fixed order.
 constexpr int GB_BM = 128, GB_BK = 16, GB_THREADS = 256;
-constexpr int kGemmMinB = 8;
+constexpr int kGemmMinB = 33;  // below, passes of gemv_kernel over 8 trajectories: n = 30,000 8 in 0.65 ms, 32 in
+                               // 2.6; one tile of 64 takes 3.1 ms however few of it are used
 
 // Row strides are padded (130 floats, GB_BN + 2 pairs) so that the transposing stores of a
 // warp (8 rows or trajectories x 4 k-quads) fall into distinct banks, while every row stays
@@ -681,9 +647,23 @@ static SplitPlan gemm_plan(const nf_operator *op, int B) {
     return p;
 }
 
-static bool use_gemm(const nf_operator *op, int B) { return op->path == NF_DENSE_FP32 && B >= kGemmMinB; }
+// Small planes give the GEMM too few tiles (12 CTAs at n = 1,500: 90 us per sum of 64 trajectories).
+static bool use_gemm(const nf_operator *op, int B) {
+    return op->path == NF_DENSE_FP32 && B >= kGemmMinB && op->n_pad >= 3072;
+}
+
+template <int NB>
+static cudaError_t sym_gemv_attrs() {
+    const int smem = (int)(sym_smem_floats<NB>(SB) * sizeof(float));
+    cudaError_t e = cudaFuncSetAttribute(gemv_sym_kernel<NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemv_sym_kernel<NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e;
+}
 
 nf_status dense_init_attrs() {
+    NF_CUDA_TRY(sym_gemv_attrs<1>());
+    NF_CUDA_TRY(sym_gemv_attrs<2>());
+    NF_CUDA_TRY(sym_gemv_attrs<4>());
     NF_CUDA_TRY(cudaFuncSetAttribute(gemm_fp32_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sizeof(GemmSmem<128>)));
     NF_CUDA_TRY(cudaFuncSetAttribute(gemm_fp32_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -694,9 +674,9 @@ nf_status dense_init_attrs() {
 SplitPlan dense_plan(nf_operator *op) {
     int res = 0;
     if (op->path == NF_DENSE_FP32)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, gemv_fp32_kernel, DG_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, gemv_kernel<1, false>, DG_THREADS, 0);
     else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, gemv_bf16x2_kernel, DG_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, gemv_kernel<1, true>, DG_THREADS, 0);
     return plan_splits(op->n_pad, DG_ROWS, DG_TILE, std::max(res, 1));
 }
 
@@ -711,19 +691,94 @@ size_t dense_sym_entries(int64_t n_pad) {
     return (size_t)(nb * (nb + 1) / 2) * SB * SB;
 }
 
+// CTAs per block pair of the symmetric GEMV: enough for one and a half waves of two CTAs per SM, at
+// most 8 (a portable cluster).  Per RK4 stage, one CTA per pair before / now: n = 4,000 38.9 /
+// 11.0 us, 8,000 81.8 / 27.1, 16,000 104.7 / 97.6; from about 465 pairs (n = 30,000) one CTA per
+// pair streams at the HBM limit and the exchange only costs (292.8 us with one, 302.1 with four).
+static int sym_slices(int64_t pairs) {
+    int S = 1;
+    while (S < 8 && pairs * S < 3 * (int64_t)num_sms()) S *= 2;
+    return S;
+}
+
+template <int NB, bool HL>
+static cudaError_t launch_sym_gemv(nf_operator *op, int B, int b0, cudaStream_t s) {
+    const int64_t nb = op->n_pad / SB, pairs = nb * (nb + 1) / 2;
+    const int S = sym_slices(pairs), rows = SB / S;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)pairs, (unsigned)S, 1);
+    cfg.blockDim = dim3(SYM_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = sym_smem_floats<NB>(rows) * sizeof(float);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2]{};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = (unsigned)S;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = op->profile ? 1 : 2;
+    return cudaLaunchKernelEx(&cfg, gemv_sym_kernel<NB, HL>,
+                              HL ? static_cast<const void *>(op->Whi) : static_cast<const void *>(op->W32),
+                              (const float *)op->g, (const float *)op->rs, op->n_pad, B, b0, rows, op->partial);
+}
+
+template <bool HL>
+static nf_status launch_sym_gemvs(nf_operator *op, int B, cudaStream_t s) {
+    for (int b = 0; b < B;) {  // 3 or 4 trajectories as 4, then 2, then 1
+        const int left = B - b;
+        if (left >= 3) {
+            NF_CUDA_TRY((launch_sym_gemv<4, HL>(op, B, b, s)));
+            b += 4;
+        } else if (left == 2) {
+            NF_CUDA_TRY((launch_sym_gemv<2, HL>(op, B, b, s)));
+            b += 2;
+        } else {
+            NF_CUDA_TRY((launch_sym_gemv<1, HL>(op, B, b, s)));
+            b += 1;
+        }
+    }
+    return NF_OK;
+}
+
+template <bool HL>
+static nf_status launch_gemvs(nf_operator *op, int B, const SplitPlan &pl, cudaStream_t s) {
+    const dim3 grid((unsigned)pl.row_blocks, (unsigned)pl.splits);
+    const void *W0 = HL ? static_cast<const void *>(op->Whi) : static_cast<const void *>(op->W32);
+    auto go = [&](auto kernel, int b) {
+        return launch_dependent(kernel, grid, DG_THREADS, 0, s, !op->profile, W0, (const uint16_t *)op->Wlo,
+                                (const float *)op->g, op->n_pad, B, b, pl.jchunk, op->partial);
+    };
+    for (int b = 0; b < B;) {
+        const int left = B - b;
+        if (left >= 8) {
+            NF_CUDA_TRY(go(gemv_kernel<8, HL>, b));
+            b += 8;
+        } else if (left >= 4) {
+            NF_CUDA_TRY(go(gemv_kernel<4, HL>, b));
+            b += 4;
+        } else if (left == 3) {
+            NF_CUDA_TRY(go(gemv_kernel<3, HL>, b));
+            b += 3;
+        } else if (left == 2) {
+            NF_CUDA_TRY(go(gemv_kernel<2, HL>, b));
+            b += 2;
+        } else {
+            NF_CUDA_TRY(go(gemv_kernel<1, HL>, b));
+            b += 1;
+        }
+    }
+    return NF_OK;
+}
+
 nf_status launch_dense_gemv(nf_operator *op, int B, cudaStream_t s, int *splits_out) {
     if (op->path == NF_DENSE_SYM_FP32 || op->path == NF_DENSE_SYM_BF16X2) {
-        const int64_t nb = op->n_pad / SB;
-        for (int b = 0; b < B; ++b) {
-            if (op->path == NF_DENSE_SYM_FP32)
-                gemv_sym_fp32_kernel<<<(unsigned)(nb * (nb + 1) / 2), SYM_THREADS, 0, s>>>(op->W32, op->g, op->n_pad,
-                                                                                         B, b, op->partial);
-            else
-                gemv_sym_bf16x2_kernel<<<(unsigned)(nb * (nb + 1) / 2), SYM_THREADS, 0, s>>>(
-                    reinterpret_cast<const uint4 *>(op->Whi), op->g, op->rs, op->n_pad, B, b, op->partial);
-            NF_CUDA_TRY(cudaGetLastError());
-        }
-        *splits_out = (int)nb;
+        if (op->path == NF_DENSE_SYM_FP32)
+            NF_TRY(launch_sym_gemvs<false>(op, B, s));
+        else
+            NF_TRY(launch_sym_gemvs<true>(op, B, s));
+        *splits_out = (int)(op->n_pad / SB);
         return NF_OK;
     }
     if (use_gemm(op, B)) {
@@ -742,15 +797,10 @@ nf_status launch_dense_gemv(nf_operator *op, int B, cudaStream_t s, int *splits_
         return NF_OK;
     }
     const SplitPlan pl = dense_plan(op);
-    dim3 grid((unsigned)pl.row_blocks, (unsigned)pl.splits);
-    for (int b = 0; b < B; ++b) {
-        if (op->path == NF_DENSE_FP32)
-            gemv_fp32_kernel<<<grid, DG_THREADS, 0, s>>>(op->W32, op->g, op->n_pad, B, b, pl.jchunk, op->partial);
-        else
-            gemv_bf16x2_kernel<<<grid, DG_THREADS, 0, s>>>(op->Whi, op->Wlo, op->g, op->n_pad, B, b, pl.jchunk,
-                                                           op->partial);
-        NF_CUDA_TRY(cudaGetLastError());
-    }
+    if (op->path == NF_DENSE_FP32)
+        NF_TRY(launch_gemvs<false>(op, B, pl, s));
+    else
+        NF_TRY(launch_gemvs<true>(op, B, pl, s));
     *splits_out = pl.splits;
     return NF_OK;
 }

@@ -62,6 +62,20 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// ------------------------------------------------------------------ thread-block clusters
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// This CTA's shared variable `p` as cluster CTA `rank` holds it.
+__device__ __forceinline__ float ld_cluster(const float *p, uint32_t rank) {
+    float v;
+    asm volatile("{\n\t.reg .u32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.f32 %0, [a];\n\t}"
+                 : "=f"(v)
+                 : "r"(smem_u32(p)), "r"(rank)
+                 : "memory");
+    return v;
+}
+
 // Block pair of CTA t over node blocks, enumerated as (0,0), (0,1), (1,1), (0,2), ...  An FP32
 // root, then integer corrections: the FP64 root this replaces cost every CTA 1.6 us of the SM's
 // FP64 pipe (two lanes per clock), 5 % of a sum at n = 100,000 and 12 % at 20,000.
