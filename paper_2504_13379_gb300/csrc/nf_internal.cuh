@@ -307,7 +307,11 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits);
 // matrix-free / dense nonlocal launches (g must hold q f(U) / f(U) for B trajectories)
 nf_status mf_init_attrs();
 nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaStream_t s);
-SplitPlan mf_plan(nf_operator *op);     // column splits of the multi-trajectory matrix-free launches
+SplitPlan mf_plan(nf_operator *op);     // column splits of the packed pair kernel
+SplitPlan multi_plan(const nf_operator *op);  // of the multi-trajectory pair kernel
+nf_status launch_multi(nf_operator *op, int B, int b0, cudaStream_t s);
+nf_status multi_init_attrs();
+void class_limits(const nf_operator *op, float *tail, float *skip);  // tile classes (nf_sym.cu)
 int mf_splits(nf_operator *op, int B);  // partial-sum slots of a matrix-free launch over B trajectories
 int mf_form(const nf_kernel &k);         // pair form of a kernel (nf_operator::form)
 float mf_unit(const nf_operator *op);    // stored coordinates per unit of the caller's

@@ -4,11 +4,13 @@
 // Pair kernel.  I[b, i] = sum_j w(|x_i - x_j|) g[b, j], g = q o f(U) (FP32), with the
 // Mexican-hat kernel w(r) = A1 exp(-r^2/s1^2) - A2 exp(-r^2/s2^2).  Work is split
 // into items (row block, column split): each warp owns R rows (coordinates in
-// registers); its lanes stride over the columns of the split; column tiles of
-// MF_TJ nodes (x, y, z and the NB trajectories' g values) are staged into shared
-// memory by the TMA bulk-copy unit, double buffered on mbarriers.  Per pair:
-// 3 FADD + FMUL + 2 FFMA (r^2), 2 FMUL (exponent scaling), 2 MUFU.EX2, and 2 FFMA
-// (NB = 1: separate e1 and e2 accumulators) or FMUL + FFMA + NB FFMA (NB > 1).
+// registers); its lanes stride over the columns of the split; column tiles are staged
+// into shared memory by the TMA bulk-copy unit, double buffered on mbarriers.  The scalar
+// kernel below serves the allocation-free call (NB = 1), whose nodes are in the caller's order,
+// and groups of exactly 16 trajectories (NB = 16), where the packed kernel of nf_multi.cu spills
+// its 64 accumulators (n = 20,000: 544 against 584 us per sum).  Per pair 3 FADD + FMUL + 2 FFMA
+// (r^2), 2 FMUL (exponent scaling), 2 MUFU.EX2, and 2 FFMA (NB = 1: separate e1 and e2
+// accumulators) or FMUL + FFMA + NB FFMA.
 // Each warp reduces its rows with shuffles and writes one partial sum per
 // (split, trajectory, row); the stage kernel (or the reduce kernel) adds the
 // splits in a fixed order, so results are deterministic.
@@ -631,14 +633,9 @@ static nf_status mf_init_attrs_device() {
     NF_TRY(dense_init_attrs());
     NF_TRY(sym_init_attrs());
     NF_TRY(adj_init_attrs());
+    NF_TRY(multi_init_attrs());
     NF_CUDA_TRY((set_mf_attr<1, 2>()));
-    NF_CUDA_TRY((set_mf_attr<2, 2>()));
-    NF_CUDA_TRY((set_mf_attr<4, 2>()));
-    NF_CUDA_TRY((set_mf_attr<8, 2>()));
     NF_CUDA_TRY((set_mf_attr<1, 4>()));
-    NF_CUDA_TRY((set_mf_attr<2, 4>()));
-    NF_CUDA_TRY((set_mf_attr<4, 4>()));
-    NF_CUDA_TRY((set_mf_attr<8, 4>()));
     NF_CUDA_TRY((set_mf_attr<16, 2>()));
     NF_CUDA_TRY((set_mf_attr<16, 4>()));
     return NF_OK;
@@ -797,7 +794,8 @@ static bool use_sym(const nf_operator *op) {
 }
 
 int mf_splits(nf_operator *op, int B) {
-    return (B <= kSymMaxB && use_sym(op)) ? sym_slots(op) : mf_plan(op).splits;
+    if (B <= kSymMaxB && use_sym(op)) return sym_slots(op);
+    return B == 1 ? mf_plan(op).splits : multi_plan(op).splits;
 }
 
 static SplitPlan variant_plan(int64_t n_pad, int v) {
@@ -829,7 +827,7 @@ void mf_launch_shape(nf_operator *op, int *R, int *TJ, int *splits) {
     *splits = sym_slots(op);
 }
 
-// Rows per warp of the scalar multi-trajectory kernel (2 or 4 are instantiated).
+// Rows per warp of the scalar kernel (2 or 4 are instantiated).
 static int mf_rows_per_warp(int64_t n_pad) { return n_pad >= 16384 ? 4 : 2; }
 
 // Time the symmetric kernel's node blocks (1,024, or 512 where those give too few CTAs) once on
@@ -1028,51 +1026,27 @@ nf_status launch_mf_pair(nf_operator *op, int B, cudaStream_t s, int *splits_out
         }
         return NF_OK;
     }
-    if (B == 1) {  // a small node set: the packed kernel over (row block, column split) items
+    if (B == 1) {  // the packed kernel over (row block, column split) items
         const SplitPlan pl = mf_plan(op);
         NF_TRY(launch_mf_packed(op, 1, 0, 1, pl, s));
         *splits_out = pl.splits;
         return NF_OK;
     }
-    // the column splits (and so the partial-sum layout) come from the packed kernel's
-    // plan; the scalar multi-trajectory kernels block rows their own way over the same splits
-    const SplitPlan pl = mf_plan(op);
-    const int R = mf_rows_per_warp(op->n_pad);
-    SplitPlan spl = pl;
-    spl.rows_per_block = MF_WARPS * R;
-    spl.row_blocks = op->n_pad / spl.rows_per_block;
-    int b = 0;
-    auto run = [&](int nb) -> nf_status {
-        const int groups = (B - b) / nb;
-        if (groups <= 0) return NF_OK;
-        nf_status st = NF_OK;
-        if (nb == 1) {
-            st = launch_mf_packed(op, B, b, groups, pl, s);
-        } else if (R == 4) {
-            switch (nb) {
-                case 16: st = launch_mf_group<16, 4>(op, B, b, groups, spl, s); break;
-                case 8: st = launch_mf_group<8, 4>(op, B, b, groups, spl, s); break;
-                case 4: st = launch_mf_group<4, 4>(op, B, b, groups, spl, s); break;
-                default: st = launch_mf_group<2, 4>(op, B, b, groups, spl, s); break;
-            }
-        } else {
-            switch (nb) {
-                case 16: st = launch_mf_group<16, 2>(op, B, b, groups, spl, s); break;
-                case 8: st = launch_mf_group<8, 2>(op, B, b, groups, spl, s); break;
-                case 4: st = launch_mf_group<4, 2>(op, B, b, groups, spl, s); break;
-                default: st = launch_mf_group<2, 2>(op, B, b, groups, spl, s); break;
-            }
-        }
-        b += groups * nb;
-        return st;
-    };
-    NF_TRY(run(16));
-    NF_TRY(run(8));
-    NF_TRY(run(4));
-    NF_TRY(run(2));
-    NF_TRY(run(1));
+    // several: groups of exactly 16 on the scalar kernel, the rest on the packed one, over the same
+    // column splits
+    SplitPlan pl = multi_plan(op);
     *splits_out = pl.splits;
-    return NF_OK;
+    const int full = B / 16;
+    if (full > 0) {
+        const int R = mf_rows_per_warp(op->n_pad);
+        pl.rows_per_block = MF_WARPS * R;
+        pl.row_blocks = op->n_pad / pl.rows_per_block;
+        if (R == 4)
+            NF_TRY((launch_mf_group<16, 4>(op, B, 0, full, pl, s)));
+        else
+            NF_TRY((launch_mf_group<16, 2>(op, B, 0, full, pl, s)));
+    }
+    return B > 16 * full ? launch_multi(op, B, 16 * full, s) : NF_OK;
 }
 
 // Launch plan of launch_mf_pair_single: at most max_splits column splits.

@@ -99,7 +99,7 @@ float mf_period(const nf_operator *op) { return op->kp.period > 0.f ? op->kp.per
 //   tail: M >= 2: |c_i| e1 / e2 = |A1 / A2| 2^(-(M - 1) r^2) < 2^-26 (c_i carries the row
 //         factors), half a unit for rounding; general form with s1 <= s2: e1 flushes as above;
 //         one Gaussian: no tail.
-static void class_limits(const nf_operator *op, float *tail, float *skip) {
+void class_limits(const nf_operator *op, float *tail, float *skip) {
     const nf_kernel &k = op->kp;
     const double k2 = ((double)k.s1 * k.s1) / ((double)k.s2 * k.s2);
     const double none = 126.0 + 4.0 + 1.0;
