@@ -371,10 +371,22 @@ class GroupedOperator(Operator):
         return out
 
 
-def _per_traj(v, B, device):
+def _per_traj(v, B, device, op):
+    """Per-trajectory parameter array of a call on ``op``.  A number's array is kept on the operator
+    (at most 16, by value, count and stream): repeated calls skip an allocation and a fill
+    launch each, and find the captured RK4 step of the call before, which names the arrays."""
     if isinstance(v, torch.Tensor):
         return v.to(device=device, dtype=torch.float32).contiguous().expand(B).contiguous()
-    return torch.full((B,), float(v), dtype=torch.float32, device=device)
+    kept = op.__dict__.setdefault("_consts", {})
+    key = (float(v), B, torch.cuda.current_stream(device).cuda_stream)
+    t = kept.get(key)
+    if t is None:
+        t = torch.full((B,), float(v), dtype=torch.float32, device=device)
+        if not torch.cuda.is_current_stream_capturing():  # a capture's memory is not ours to keep
+            if len(kept) >= 16:
+                kept.clear()
+            kept[key] = t
+    return t
 
 
 def nf_nonlocal_apply(op: Operator, u: torch.Tensor, beta, theta, out: torch.Tensor | None = None) -> torch.Tensor:
@@ -385,7 +397,7 @@ def nf_nonlocal_apply(op: Operator, u: torch.Tensor, beta, theta, out: torch.Ten
     else:
         u2 = u if u.dim() == 2 else u.view(1, -1)
         B = u2.shape[0]
-    be, th = _per_traj(beta, B, u.device), _per_traj(theta, B, u.device)
+    be, th = _per_traj(beta, B, u.device, op), _per_traj(theta, B, u.device, op)
     I = out if out is not None else torch.empty_like(u2)
     _check(lib().nf_nonlocal_apply(op.handle, _dptr(u2, torch.float32, "u"), B, _dptr(be, torch.float32, "beta"),
                                    _dptr(th, torch.float32, "theta"), _dptr(I, torch.float32, "I"), _stream(u)))
@@ -457,7 +469,7 @@ def nf_rk4_advance(op: Operator, u: torch.Tensor, t0: float, dt: float, nsteps: 
     else:
         u2 = u if u.dim() == 2 else u.view(1, -1)
         B = u2.shape[0]
-    be, th = _per_traj(beta, B, u.device), _per_traj(theta, B, u.device)
+    be, th = _per_traj(beta, B, u.device, op), _per_traj(theta, B, u.device, op)
     f = C.byref(forcing._struct()) if forcing is not None else None
     cp = _dptr(ckpt, torch.float32, "ckpt") if ckpt is not None else None
     _check(lib().nf_rk4_advance(op.handle, _dptr(u2, torch.float32, "u"), B, float(t0), float(dt), int(nsteps),
@@ -480,7 +492,7 @@ def nf_field_advance(op: Operator, u: torch.Tensor, dt: float, nsteps: int, beta
     u2 = u if u.dim() == 2 else u.view(1, -1)
     B = u2.shape[0]
     s2 = None if s is None else (s if s.dim() == 2 else s.view(1, -1))
-    be, th = _per_traj(beta, B, u.device), _per_traj(theta, B, u.device)
+    be, th = _per_traj(beta, B, u.device, op), _per_traj(theta, B, u.device, op)
     m = _Model(MODEL_DEPRESSION if s is not None else MODEL_FIELD, int(rate), float(a), float(b), float(tau),
                float(beta_d))
     integ = {"rk4": 0, "ab5": 1}[integrator]
@@ -497,7 +509,7 @@ def nf_adjoint(op: Operator, ckpt: torch.Tensor, C_every: int, t0: float, dt: fl
     """Discrete RK4 adjoint: returns (dL/du0 (B x n), dL/d(A1,s1,A2,s2) (B x 4))."""
     lam = lambda_T if lambda_T.dim() == 2 else lambda_T.view(1, -1)
     B, n = lam.shape
-    be, th = _per_traj(beta, B, lam.device), _per_traj(theta, B, lam.device)
+    be, th = _per_traj(beta, B, lam.device, op), _per_traj(theta, B, lam.device, op)
     gu = torch.empty_like(lam)
     gk = torch.empty((B, 4), dtype=torch.float32, device=lam.device)
     f = C.byref(forcing._struct()) if forcing is not None else None
