@@ -48,38 +48,31 @@ int num_sms() {
 }
 
 // ---------------------------------------------------------------- workspace
-nf_status ensure_workspace(nf_operator *op, int B, int splits) {
+// One allocation holds partial, g and (state) U, ks, us: a new operator's first call pays for one
+// cudaMalloc instead of five.  It grows to the largest of each part asked for so far.
+nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state) {
     const size_t need_p = (size_t)splits * B * op->n_pad;
     const size_t need_g = (fused_fits(op, B) ? 2 : 1) * (size_t)B * op->n_pad;  // fused stages alternate
-    const size_t need_s = (size_t)B * op->n;
-    // captured graphs hold workspace pointers: drop them before anything moves
-    if (need_p > op->partial_cap || need_g > op->g_cap || need_s > op->state_cap) destroy_graphs(op);
-    if (need_p > op->partial_cap) {
-        if (op->partial) NF_CUDA_TRY(cudaFree(op->partial));
-        op->partial = nullptr;
-        op->partial_cap = 0;
-        NF_CUDA_TRY(cudaMalloc(&op->partial, need_p * sizeof(float)));
-        op->partial_cap = need_p;
-    }
-    if (need_g > op->g_cap) {
-        if (op->g) NF_CUDA_TRY(cudaFree(op->g));
-        op->g = nullptr;
-        op->g_cap = 0;
-        NF_CUDA_TRY(cudaMalloc(&op->g, need_g * sizeof(float)));
-        NF_CUDA_TRY(cudaMemset(op->g, 0, need_g * sizeof(float)));  // padding columns stay zero
-        op->g_cap = need_g;
-    }
-    if (need_s > op->state_cap) {
-        if (op->U) NF_CUDA_TRY(cudaFree(op->U));
-        if (op->ks) NF_CUDA_TRY(cudaFree(op->ks));
-        if (op->us) NF_CUDA_TRY(cudaFree(op->us));
-        op->U = op->ks = op->us = nullptr;
-        op->state_cap = 0;
-        if (op->perm) NF_CUDA_TRY(cudaMalloc(&op->us, need_s * sizeof(float)));
-        NF_CUDA_TRY(cudaMalloc(&op->U, need_s * sizeof(float)));
-        NF_CUDA_TRY(cudaMalloc(&op->ks, need_s * sizeof(float)));
-        op->state_cap = need_s;
-    }
+    const size_t need_s = state ? (size_t)B * op->n : 0;
+    if (need_p <= op->partial_cap && need_g <= op->g_cap && need_s <= op->state_cap) return NF_OK;
+    destroy_graphs(op);  // captured graphs hold workspace pointers
+    auto part = [](size_t have, size_t need) { return (std::max(have, need) + 63) / 64 * 64; };  // 256-byte steps
+    const size_t cp = part(op->partial_cap, need_p), cg = part(op->g_cap, need_g), cs = part(op->state_cap, need_s);
+    const int states = op->perm ? 3 : 2;
+    if (op->partial) NF_CUDA_TRY(cudaFree(op->partial));
+    op->partial = op->g = op->U = op->ks = op->us = nullptr;
+    op->partial_cap = op->g_cap = op->state_cap = 0;
+    float *mem = nullptr;
+    NF_CUDA_TRY(cudaMalloc(&mem, (cp + cg + states * cs) * sizeof(float)));
+    op->partial = mem;
+    op->g = mem + cp;
+    op->U = op->g + cg;
+    op->ks = op->U + cs;
+    if (op->perm) op->us = op->ks + cs;
+    NF_CUDA_TRY(cudaMemset(op->g, 0, cg * sizeof(float)));  // padding columns stay zero
+    op->partial_cap = cp;
+    op->g_cap = cg;
+    op->state_cap = cs;
     return NF_OK;
 }
 
@@ -368,19 +361,18 @@ nf_status nf_operator_create(const float *x, const float *q, int64_t n, nf_kerne
         cudaError_t _e = (expr);                                                            \
         if (_e != cudaSuccess) return cleanup(cuda_fail(_e, #expr, __FILE__, __LINE__));    \
     } while (0)
-    CREATE_TRY(cudaMalloc(&op->x4, op->n_pad * sizeof(float4)));
-    CREATE_TRY(cudaMalloc(&op->q, op->n_pad * sizeof(float)));
     CREATE_TRY(cudaMalloc(&op->step_ctr, 64));
     CREATE_TRY(cudaMemsetAsync(op->step_ctr, 0, 64, s));
     op->done_ctr = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(op->step_ctr) + 16);
     op->err = reinterpret_cast<int *>(reinterpret_cast<char *>(op->step_ctr) + 32);
     op->t0_dev = reinterpret_cast<double *>(reinterpret_cast<char *>(op->step_ctr) + 40);
     if (path == NF_MATRIX_FREE) {
-        CREATE_TRY(cudaMalloc(&op->xyz, 3 * op->n_pad * sizeof(float)));
         nf_status st = mf_build_nodes(op, x, q, s);
         if (st == NF_OK) st = mf_autotune(op, s);
         if (st != NF_OK) return cleanup(st);
     } else {
+        CREATE_TRY(cudaMalloc(&op->x4, op->n_pad * sizeof(float4)));
+        CREATE_TRY(cudaMalloc(&op->q, op->n_pad * sizeof(float)));
         pack_nodes_kernel<<<(unsigned)ceil_div(op->n_pad, 256), 256, 0, s>>>(x, q, n, op->n_pad, op->x4, op->q);
         CREATE_TRY(cudaGetLastError());
         const size_t entries = (size_t)op->n_pad * (size_t)op->n_pad;
@@ -409,26 +401,28 @@ nf_status nf_operator_destroy(nf_operator *op) {
     destroy_graphs(op);
     destroy_group(op);
     destroy_prof_ring(op);
-    cudaFree(op->x4);
-    cudaFree(op->xyz);
-    cudaFree(op->perm);
-    cudaFree(op->rg);  // with rw, pc, pe, tc, te
+    if (op->path == NF_MATRIX_FREE) {
+        cudaFree(op->rg);  // with every other node array
+    } else {
+        cudaFree(op->x4);
+        cudaFree(op->q);
+    }
     cudaFree(op->cull_pairs);
     cudaFree(op->cull_ptr);
     cudaFree(op->cull_slots);
     cudaFree(op->adj_pairs);
     cudaFree(op->adj_ptr);
     cudaFree(op->adj_slots);
-    cudaFree(op->q);
     cudaFree(op->W32);
     cudaFree(op->Whi);
     cudaFree(op->Wlo);
     cudaFree(op->rs);
-    cudaFree(op->partial);
-    cudaFree(op->g);
-    cudaFree(op->U);
-    cudaFree(op->ks);
-    cudaFree(op->us);
+    if (op->path == NF_GROUPED) {
+        cudaFree(op->U);
+        cudaFree(op->ks);
+    } else {
+        cudaFree(op->partial);  // with g, U, ks, us
+    }
     cudaFree(op->step_ctr);
     delete op;
     return NF_OK;
@@ -459,7 +453,7 @@ nf_status nf_nonlocal_apply(nf_operator *op, const float *u, int B, const float 
         NF_TRY(tc_prep(op, u, beta, theta, false, 0, s));
         return tc_launch(op, 0, 0, I, nullptr, beta, theta, 0.0, 0, nullptr, 1, s);
     }
-    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B)));
+    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B), false));
     NF_TRY(launch_prep_g(op, u, B, beta, theta, false, s));
     if (fused_fits(op, B)) return fused_apply(op, B, I, s);
     int splits = 1;

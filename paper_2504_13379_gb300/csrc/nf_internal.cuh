@@ -139,10 +139,10 @@ struct PerTag {
     static constexpr bool value = P;
 };
 
-// A loop bound known at compile time (full node blocks), interchangeable with a runtime int
-// bound (the last, partial block) in templated loops.
+// An integer known at compile time, as an argument.
 template <int V>
 struct CInt {
+    static constexpr int value = V;
     __device__ constexpr operator int() const { return V; }
 };
 
@@ -302,7 +302,7 @@ SplitPlan plan_splits(int64_t n_pad, int rows_per_block, int tile_cols, int resi
 void launch_validate_indices(const int32_t *idx, int64_t cnt, int64_t n, int *flag, cudaStream_t s);
 void launch_exclusive_scan(const int32_t *in, int64_t len, int32_t *out, cudaStream_t s);
 
-nf_status ensure_workspace(nf_operator *op, int B, int splits);
+nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state = true);
 
 // matrix-free / dense nonlocal launches (g must hold q f(U) / f(U) for B trajectories)
 nf_status mf_init_attrs();

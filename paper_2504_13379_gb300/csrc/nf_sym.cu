@@ -315,6 +315,31 @@ __global__ void row_bitonic_kernel(unsigned long long *__restrict__ keys, int64_
     }
 }
 
+// All steps of the network that stay within blocks of SORT_BLK keys, in shared memory: block
+// sizes kk0 .. kk1, partner distances below SORT_BLK (a sort of 131,072 keys takes 28 launches
+// instead of 153).
+constexpr int SORT_BLK = 2048;
+__global__ void __launch_bounds__(SORT_BLK / 2)
+row_bitonic_local_kernel(unsigned long long *__restrict__ keys, int blk, int64_t kk0, int64_t kk1) {
+    __shared__ unsigned long long k[SORT_BLK];
+    const int64_t base = (int64_t)blockIdx.x * blk;
+    for (int i = threadIdx.x; i < blk; i += blockDim.x) k[i] = keys[base + i];
+    __syncthreads();
+    for (int64_t kk = kk0; kk <= kk1; kk <<= 1)
+        for (int jj = (int)min(kk, (int64_t)blk) >> 1; jj > 0; jj >>= 1) {
+            for (int t = threadIdx.x; t < blk / 2; t += blockDim.x) {
+                const int i = (t / jj) * 2 * jj + t % jj, l = i + jj;
+                const unsigned long long a = k[i], b = k[l];
+                if ((a > b) == (((base + i) & kk) == 0)) {
+                    k[i] = b;
+                    k[l] = a;
+                }
+            }
+            __syncthreads();
+        }
+    for (int i = threadIdx.x; i < blk; i += blockDim.x) keys[base + i] = k[i];
+}
+
 // Node arrays in Hilbert order.  Padding repeats the last node (so that it widens no box) with
 // q = 0 (so that it contributes nothing).
 __global__ void pack_sorted_kernel(const float *__restrict__ x, const float *__restrict__ q,
@@ -339,24 +364,33 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     op->form = mf_form(k);
     int64_t m = 1;
     while (m < n_pad) m <<= 1;
-    NF_CUDA_TRY(cudaMalloc(&op->perm, sizeof(int) * n_pad));
+    // One allocation for all node arrays, 16-byte types first, and the bounding box.  The sort's keys
+    // (m < 2 n_pad of 8 bytes) take rg's place until sym_static_kernel writes it.
     const int64_t np = n_pad / kPassRows, nt = n_pad / kTileCols;
     unsigned char *mem = nullptr;
-    NF_CUDA_TRY(cudaMalloc(&mem, sizeof(float4) * (n_pad + 2 * np + 2 * nt) + sizeof(float2) * n_pad));
+    NF_CUDA_TRY(cudaMalloc(&mem, sizeof(float4) * (2 * n_pad + 2 * np + 2 * nt) + sizeof(float2) * n_pad +
+                                     (4 * sizeof(float) + sizeof(int)) * n_pad + 64));
     op->rg = reinterpret_cast<float4 *>(mem);
-    op->pc = op->rg + n_pad;
+    op->x4 = op->rg + n_pad;
+    op->pc = op->x4 + n_pad;
     op->pe = op->pc + np;
     op->tc = op->pe + np;
     op->te = op->tc + nt;
-    op->rw = reinterpret_cast<float2 *>(op->te + nt);
-    unsigned long long *keys = nullptr;
-    NF_CUDA_TRY(cudaMalloc(&keys, sizeof(unsigned long long) * m + 64));
-    float *box = reinterpret_cast<float *>(keys + m);
+    op->xyz = reinterpret_cast<float *>(op->te + nt);  // n_pad is a multiple of 1024: each array stays aligned
+    op->q = op->xyz + 3 * n_pad;
+    op->rw = reinterpret_cast<float2 *>(op->q + n_pad);
+    op->perm = reinterpret_cast<int *>(op->rw + n_pad);
+    unsigned long long *keys = reinterpret_cast<unsigned long long *>(op->rg);
+    float *box = reinterpret_cast<float *>(op->perm + n_pad);
     row_bbox_kernel<<<1, 1024, 0, s>>>(x, n, box);
     row_key_kernel<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(x, n, m, box, keys);
-    for (int64_t kk = 2; kk <= m; kk <<= 1)
-        for (int64_t jj = kk >> 1; jj > 0; jj >>= 1)
+    const int blk = (int)std::min<int64_t>(m, SORT_BLK);
+    row_bitonic_local_kernel<<<(unsigned)(m / blk), SORT_BLK / 2, 0, s>>>(keys, blk, 2, blk);
+    for (int64_t kk = 2 * blk; kk <= m; kk <<= 1) {
+        for (int64_t jj = kk >> 1; jj >= blk; jj >>= 1)
             row_bitonic_kernel<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(keys, m, jj, kk);
+        row_bitonic_local_kernel<<<(unsigned)(m / blk), SORT_BLK / 2, 0, s>>>(keys, blk, kk, kk);
+    }
     pack_sorted_kernel<<<(unsigned)ceil_div(n_pad, 256), 256, 0, s>>>(x, q, keys, n, n_pad, mf_unit(op), op->x4,
                                                                      op->xyz, op->q, op->perm);
     // the threshold of the expanded form in the stored units
@@ -370,7 +404,6 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     if (e == cudaSuccess) e = cudaMemcpyAsync(hbox, box, sizeof(hbox), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     op->planar = (e == cudaSuccess && hbox[2] == hbox[5]) ? 1 : 0;  // one z for every node
-    cudaFree(keys);
     if (e != cudaSuccess) return cuda_fail(e, "node order", __FILE__, __LINE__);
     return NF_OK;
 }
