@@ -78,6 +78,27 @@ adj_sym_kernel(SymNodes nd, const float *__restrict__ nu_all, const float *__res
 
     bool bad = false, live = false;
     for (int k = tid; k < BLK / 4; k += AS_THREADS) {
+        cp_async16(xs + 4 * k, nd.xyz + cbase + 4 * k);
+        cp_async16(ys + 4 * k, nd.xyz + n_pad + cbase + 4 * k);
+        cp_async16(zs + 4 * k, nd.xyz + 2 * n_pad + cbase + 4 * k);
+    }
+    for (int k = tid; k < BLK; k += AS_THREADS) cp_async16(rg + k, nd.rg + rbase + k);
+    for (int k = tid; k < BLK / 2; k += AS_THREADS) cp_async16(rw + 2 * k, nd.rw + rbase + 2 * k);
+    for (int k = tid; k < BLK / kPassRows; k += AS_THREADS) {
+        cp_async16(pc + k, nd.pc + rbase / kPassRows + k);
+        cp_async16(pe + k, nd.pe + rbase / kPassRows + k);
+    }
+    if (tid < NT) {
+        cp_async16(tcs + tid, nd.tc + cbase / kTileCols + tid);
+        cp_async16(tes + tid, nd.te + cbase / kTileCols + tid);
+    }
+    if (!diag)
+        for (int k = tid; k < AS_WARPS * BLK / 4; k += AS_THREADS)
+            reinterpret_cast<float4 *>(colacc)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // everything above depends on the operator alone; nu and g are written by the kernel before
+    pdl_wait();
+    pdl_trigger();
+    for (int k = tid; k < BLK / 4; k += AS_THREADS) {
         const float4 v[4] = {__ldg(reinterpret_cast<const float4 *>(nu + cbase) + k),
                              __ldg(reinterpret_cast<const float4 *>(g + cbase) + k),
                              __ldg(reinterpret_cast<const float4 *>(nu + rbase) + k),
@@ -102,26 +123,9 @@ adj_sym_kernel(SymNodes nd, const float *__restrict__ nu_all, const float *__res
             reinterpret_cast<float4 *>(out_cols)[k] = zero;
         }
         if (tid < 4) out_g[tid] = 0.f;
+        cp_async_wait_all();
         return;
     }
-    for (int k = tid; k < BLK / 4; k += AS_THREADS) {
-        cp_async16(xs + 4 * k, nd.xyz + cbase + 4 * k);
-        cp_async16(ys + 4 * k, nd.xyz + n_pad + cbase + 4 * k);
-        cp_async16(zs + 4 * k, nd.xyz + 2 * n_pad + cbase + 4 * k);
-    }
-    for (int k = tid; k < BLK; k += AS_THREADS) cp_async16(rg + k, nd.rg + rbase + k);
-    for (int k = tid; k < BLK / 2; k += AS_THREADS) cp_async16(rw + 2 * k, nd.rw + rbase + 2 * k);
-    for (int k = tid; k < BLK / kPassRows; k += AS_THREADS) {
-        cp_async16(pc + k, nd.pc + rbase / kPassRows + k);
-        cp_async16(pe + k, nd.pe + rbase / kPassRows + k);
-    }
-    if (tid < NT) {
-        cp_async16(tcs + tid, nd.tc + cbase / kTileCols + tid);
-        cp_async16(tes + tid, nd.te + cbase / kTileCols + tid);
-    }
-    if (!diag)
-        for (int k = tid; k < AS_WARPS * BLK / 4; k += AS_THREADS)
-            reinterpret_cast<float4 *>(colacc)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
     cp_async_wait_all();
     __syncthreads();
 
@@ -388,30 +392,23 @@ nf_status launch_adj_sym(nf_operator *op, const float *nu, const float *g, int B
     const float per = mf_period(op);
     float tail, skip;
     adj_limits(op, &tail, &skip);
-#define NF_ADJ_ARGS nd, nu, g, B, b, k2, k.A1, k.A2, per, tail, skip, wpart, gpart, pairs
-#define NF_ADJ_LAUNCH(RR, BB)                                                                     \
-    switch (m) {                                                                                  \
-        case 2: adj_sym_kernel<RR, 2, BB><<<grid, AS_THREADS, smem, s>>>(NF_ADJ_ARGS); break;     \
-        case 3: adj_sym_kernel<RR, 3, BB><<<grid, AS_THREADS, smem, s>>>(NF_ADJ_ARGS); break;     \
-        case 4: adj_sym_kernel<RR, 4, BB><<<grid, AS_THREADS, smem, s>>>(NF_ADJ_ARGS); break;     \
-        default: adj_sym_kernel<RR, 0, BB><<<grid, AS_THREADS, smem, s>>>(NF_ADJ_ARGS); break;    \
-    }
-    if (blk == 512) {
-        if (op->adj_r == 8) {
-            NF_ADJ_LAUNCH(8, 512)
-        } else {
-            NF_ADJ_LAUNCH(4, 512)
+    auto go = [&](auto kernel) {
+        return launch_dependent(kernel, dim3(grid), AS_THREADS, smem, s, true, nd, nu, g, B, b, k2, k.A1, k.A2, per, tail,
+                                skip, wpart, gpart, pairs);
+    };
+    auto form = [&](auto r_tag, auto blk_tag) {
+        constexpr int R = decltype(r_tag)::value, BLK = decltype(blk_tag)::value;
+        switch (m) {
+            case 2: return go(adj_sym_kernel<R, 2, BLK>);
+            case 3: return go(adj_sym_kernel<R, 3, BLK>);
+            case 4: return go(adj_sym_kernel<R, 4, BLK>);
+            default: return go(adj_sym_kernel<R, 0, BLK>);
         }
-    } else {
-        if (op->adj_r == 8) {
-            NF_ADJ_LAUNCH(8, 1024)
-        } else {
-            NF_ADJ_LAUNCH(4, 1024)
-        }
-    }
-#undef NF_ADJ_LAUNCH
-#undef NF_ADJ_ARGS
-    NF_CUDA_TRY(cudaGetLastError());
+    };
+    if (blk == 512)
+        NF_CUDA_TRY(op->adj_r == 8 ? form(CInt<8>{}, CInt<512>{}) : form(CInt<4>{}, CInt<512>{}));
+    else
+        NF_CUDA_TRY(op->adj_r == 8 ? form(CInt<8>{}, CInt<1024>{}) : form(CInt<4>{}, CInt<1024>{}));
     return NF_OK;
 }
 

@@ -66,13 +66,44 @@ struct AdjEpiArgs {
     float dt;
 };
 
-__global__ void adj_epilogue_kernel(AdjEpiArgs a) {
+// gk[b][k] += scale[k] * sum_c gpart[b][c][k] over the CTAs c of the stage's pair launch, in a fixed
+// order.  scale = (1, 2 A1 / s1^3 * r2phys, -1, -2 A2 / s2^3 * r2phys): d w / dA1 = e1,
+// d w / ds1 = 2 A1 r^2 e1 / s1^3, d w / dA2 = -e2, d w / ds2 = -2 A2 r^2 e2 / s2^3, with r^2
+// converted from exponent units.
+struct AdjScale {
+    double k[4];
+};
+
+// Epilogue of a stage (blocks 0 .. eblocks - 1: one node per thread) and the parameter sums (blocks
+// eblocks + 4 b + k), in one launch: the sums are a chain of FP64 adds that the epilogue hides.
+__global__ void __launch_bounds__(256)
+adj_epilogue_kernel(AdjEpiArgs a, int eblocks, const float *__restrict__ gpart, int64_t ncta, AdjScale sc,
+                    double *__restrict__ gk) {
+    if ((int)blockIdx.x >= eblocks) {
+        __shared__ double red[256];
+        const int out = (int)blockIdx.x - eblocks, b = out >> 2, k = out & 3;
+        const float *c = gpart + (int64_t)b * ncta * 4 + k;
+        pdl_wait();
+        double s = 0.0;
+        for (int64_t i = threadIdx.x; i < ncta; i += blockDim.x) s += (double)c[i * 4];
+        red[threadIdx.x] = s;
+        __syncthreads();
+        for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+            if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
+            __syncthreads();
+        }
+        if (threadIdx.x == 0) gk[out] += sc.k[k] * red[0];
+        return;
+    }
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)a.B * a.n) return;
-    const int b = (int)(idx / a.n);
-    const int64_t i = idx - (int64_t)b * a.n;
-    const float Wnu = sum_slots(a.wpart + (int64_t)b * a.n_pad + i, (int64_t)a.B * a.n_pad, a.slots);
+    const bool in = idx < (int64_t)a.B * a.n;
+    const int b = in ? (int)(idx / a.n) : 0;
+    const int64_t i = in ? idx - (int64_t)b * a.n : 0;
     const int64_t vi = (int64_t)b * a.n_pad + i;
+    pdl_wait();
+    pdl_trigger();
+    if (!in) return;
+    const float Wnu = sum_slots(a.wpart + (int64_t)b * a.n_pad + i, (int64_t)a.B * a.n_pad, a.slots);
     const float nu = a.nu[vi];
     const float bb = a.beta[b], th = a.theta[b];
     const float f = sigmoid_rate(a.Ucur[idx], bb, th);
@@ -95,28 +126,6 @@ __global__ void adj_epilogue_kernel(AdjEpiArgs a) {
             a.g[vi] = a.q[i] * sigmoid_rate(a.Uprev[idx], bb, th);
         }
     }
-}
-
-// gk[b][k] += scale[k] * sum_c gpart[b][c][k] over the CTAs c of the stage's pair launch,
-// one block per (b, k), fixed order.  scale = (1, 2 A1 / s1^3 * r2phys, -1, -2 A2 / s2^3 *
-// r2phys): d w / dA1 = e1, d w / ds1 = 2 A1 r^2 e1 / s1^3, d w / dA2 = -e2,
-// d w / ds2 = -2 A2 r^2 e2 / s2^3, with r^2 converted from exponent units.
-struct AdjScale {
-    double k[4];
-};
-__global__ void adj_reduce_kernel(const float *__restrict__ gpart, int64_t ncta, AdjScale sc, double *__restrict__ gk) {
-    __shared__ double red[256];
-    const int b = blockIdx.x >> 2, k = blockIdx.x & 3;
-    const float *c = gpart + (int64_t)b * ncta * 4 + k;
-    double s = 0.0;
-    for (int64_t i = threadIdx.x; i < ncta; i += blockDim.x) s += (double)c[i * 4];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if ((int)threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) gk[blockIdx.x] += sc.k[k] * red[0];
 }
 
 __global__ void adj_finish_kernel(const double *__restrict__ gk, int cnt, float *__restrict__ out) {
@@ -246,6 +255,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
         NF_CUDA_TRY(cudaMemcpyAsync(st, op->U, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
         for (int j = 0; j < cnt; ++j) {
             for (int stage = 1; stage <= 4; ++stage) {
+                if (stage == 4 && j + 1 == cnt) break;  // its sum only leads to the next segment's state
                 int splits = 1;
                 NF_TRY(launch_mf_pair(op, B, ss, &splits));
                 StageParams p{};
@@ -259,7 +269,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 p.C = 1;
                 p.splits = splits;
                 p.overlap = true;
-                p.stage_out = (stage < 4 || j + 1 < cnt) ? st + ((size_t)j * 4 + stage) * BN : nullptr;
+                p.stage_out = st + ((size_t)j * 4 + stage) * BN;
                 NF_TRY(launch_stage(op, B, p, ss));
             }
         }
@@ -316,9 +326,8 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 ea.dt = (float)dt;
                 AdjScale sc{{1.0, 2.0 * kp.A1 / ((double)kp.s1 * kp.s1 * kp.s1) * r2phys, -1.0,
                              -2.0 * kp.A2 / ((double)kp.s2 * kp.s2 * kp.s2) * r2phys}};
-                adj_reduce_kernel<<<(unsigned)(4 * B), 256, 0, s>>>(gpart, ncta_run, sc, gk);
-                adj_epilogue_kernel<<<eg, T, 0, s>>>(ea);
-                NF_CUDA_TRY(cudaGetLastError());
+                NF_CUDA_TRY(launch_dependent(adj_epilogue_kernel, dim3(eg + 4 * (unsigned)B), T, 0, s, true, ea, (int)eg,
+                                             (const float *)gpart, ncta_run, sc, gk));
             }
         }
         NF_CUDA_TRY(cudaEventRecord(side.rev[bufi], s));  // segst may now be overwritten
