@@ -377,15 +377,16 @@ def _per_traj(v, B, device, op):
     launch each, and find the captured RK4 step of the call before, which names the arrays."""
     if isinstance(v, torch.Tensor):
         return v.to(device=device, dtype=torch.float32).contiguous().expand(B).contiguous()
+    if torch.cuda.is_current_stream_capturing():  # the caller's graph keeps its own copy, in its own pool
+        return torch.full((B,), float(v), dtype=torch.float32, device=device)
     kept = op.__dict__.setdefault("_consts", {})
     key = (float(v), B, torch.cuda.current_stream(device).cuda_stream)
     t = kept.get(key)
     if t is None:
         t = torch.full((B,), float(v), dtype=torch.float32, device=device)
-        if not torch.cuda.is_current_stream_capturing():  # a capture's memory is not ours to keep
-            if len(kept) >= 16:
-                kept.clear()
-            kept[key] = t
+        if len(kept) >= 16:
+            kept.clear()
+        kept[key] = t
     return t
 
 

@@ -48,31 +48,37 @@ int num_sms() {
 }
 
 // ---------------------------------------------------------------- workspace
-// One allocation holds partial, g and (state) U, ks, us: a new operator's first call pays for one
-// cudaMalloc instead of five.  It grows to the largest of each part asked for so far.
+// partial and g share one allocation, the states U, ks, us (RK4, models, adjoint) another, so a new
+// operator's first call pays for two cudaMalloc instead of five.  Each grows to the largest of its
+// parts asked for so far; sums keep their addresses when a later call of the same width adds states.
 nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state) {
     const size_t need_p = (size_t)splits * B * op->n_pad;
     const size_t need_g = (fused_fits(op, B) ? 2 : 1) * (size_t)B * op->n_pad;  // fused stages alternate
     const size_t need_s = state ? (size_t)B * op->n : 0;
-    if (need_p <= op->partial_cap && need_g <= op->g_cap && need_s <= op->state_cap) return NF_OK;
-    destroy_graphs(op);  // captured graphs hold workspace pointers
+    const bool sums = need_p > op->partial_cap || need_g > op->g_cap, states = need_s > op->state_cap;
+    if (sums || states) destroy_graphs(op);  // captured graphs hold workspace pointers
     auto part = [](size_t have, size_t need) { return (std::max(have, need) + 63) / 64 * 64; };  // 256-byte steps
-    const size_t cp = part(op->partial_cap, need_p), cg = part(op->g_cap, need_g), cs = part(op->state_cap, need_s);
-    const int states = op->perm ? 3 : 2;
-    if (op->partial) NF_CUDA_TRY(cudaFree(op->partial));
-    op->partial = op->g = op->U = op->ks = op->us = nullptr;
-    op->partial_cap = op->g_cap = op->state_cap = 0;
-    float *mem = nullptr;
-    NF_CUDA_TRY(cudaMalloc(&mem, (cp + cg + states * cs) * sizeof(float)));
-    op->partial = mem;
-    op->g = mem + cp;
-    op->U = op->g + cg;
-    op->ks = op->U + cs;
-    if (op->perm) op->us = op->ks + cs;
-    NF_CUDA_TRY(cudaMemset(op->g, 0, cg * sizeof(float)));  // padding columns stay zero
-    op->partial_cap = cp;
-    op->g_cap = cg;
-    op->state_cap = cs;
+    if (sums) {
+        const size_t cp = part(op->partial_cap, need_p), cg = part(op->g_cap, need_g);
+        if (op->partial) NF_CUDA_TRY(cudaFree(op->partial));
+        op->partial = op->g = nullptr;
+        op->partial_cap = op->g_cap = 0;
+        NF_CUDA_TRY(cudaMalloc(&op->partial, (cp + cg) * sizeof(float)));
+        op->g = op->partial + cp;
+        NF_CUDA_TRY(cudaMemset(op->g, 0, cg * sizeof(float)));  // padding columns stay zero
+        op->partial_cap = cp;
+        op->g_cap = cg;
+    }
+    if (states) {
+        const size_t cs = part(0, need_s);
+        if (op->U) NF_CUDA_TRY(cudaFree(op->U));
+        op->U = op->ks = op->us = nullptr;
+        op->state_cap = 0;
+        NF_CUDA_TRY(cudaMalloc(&op->U, (op->perm ? 3 : 2) * cs * sizeof(float)));
+        op->ks = op->U + cs;
+        if (op->perm) op->us = op->ks + cs;
+        op->state_cap = cs;
+    }
     return NF_OK;
 }
 
@@ -417,12 +423,9 @@ nf_status nf_operator_destroy(nf_operator *op) {
     cudaFree(op->Whi);
     cudaFree(op->Wlo);
     cudaFree(op->rs);
-    if (op->path == NF_GROUPED) {
-        cudaFree(op->U);
-        cudaFree(op->ks);
-    } else {
-        cudaFree(op->partial);  // with g, U, ks, us
-    }
+    cudaFree(op->partial);  // with g
+    cudaFree(op->U);        // with ks and us
+    if (op->path == NF_GROUPED) cudaFree(op->ks);
     cudaFree(op->step_ctr);
     delete op;
     return NF_OK;
