@@ -42,7 +42,7 @@ constexpr size_t as_smem_bytes(int blk) {
 // block pairs leave the last wave of CTAs partly empty).
 template <int R, int M, int BLK>
 __global__ void __launch_bounds__(AS_THREADS, R >= 8 ? 1 : 2)
-adj_sym_kernel(SymNodes nd, const float *__restrict__ nu_all, const float *__restrict__ g_all, int B, int b, float k2,
+adj_sym_kernel(SymNodes nd, const float *nu_all, const float *g_all, int B, int b, float k2,
                float A1, float A2, float per, float lim_tail, float lim_skip, float *__restrict__ wpart,
                float *__restrict__ gpart, const int *__restrict__ pairs) {
     static_assert(M == 0 || (M >= 2 && M <= 4), "width ratio M must be 0 (general), 2, 3 or 4");
@@ -100,10 +100,9 @@ adj_sym_kernel(SymNodes nd, const float *__restrict__ nu_all, const float *__res
     pdl_wait();
     pdl_trigger();
     for (int k = tid; k < BLK / 4; k += AS_THREADS) {
-        const float4 v[4] = {__ldg(reinterpret_cast<const float4 *>(nu + cbase) + k),
-                             __ldg(reinterpret_cast<const float4 *>(g + cbase) + k),
-                             __ldg(reinterpret_cast<const float4 *>(nu + rbase) + k),
-                             __ldg(reinterpret_cast<const float4 *>(g + rbase) + k)};
+        const float4 v[4] = {
+            reinterpret_cast<const float4 *>(nu + cbase)[k], reinterpret_cast<const float4 *>(g + cbase)[k],
+            reinterpret_cast<const float4 *>(nu + rbase)[k], reinterpret_cast<const float4 *>(g + rbase)[k]};
         reinterpret_cast<float4 *>(vs)[k] = v[0];
         reinterpret_cast<float4 *>(gsm)[k] = v[1];
         reinterpret_cast<float4 *>(rnu)[k] = v[2];

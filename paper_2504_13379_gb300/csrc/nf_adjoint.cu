@@ -77,8 +77,7 @@ struct AdjScale {
 // Epilogue of a stage (blocks 0 .. eblocks - 1: one node per thread) and the parameter sums (blocks
 // eblocks + 4 b + k), in one launch: the sums are a chain of FP64 adds that the epilogue hides.
 __global__ void __launch_bounds__(256)
-adj_epilogue_kernel(AdjEpiArgs a, int eblocks, const float *__restrict__ gpart, int64_t ncta, AdjScale sc,
-                    double *__restrict__ gk) {
+adj_epilogue_kernel(AdjEpiArgs a, int eblocks, const float *gpart, int64_t ncta, AdjScale sc, double *gk) {
     if ((int)blockIdx.x >= eblocks) {
         __shared__ double red[256];
         const int out = (int)blockIdx.x - eblocks, b = out >> 2, k = out & 3;

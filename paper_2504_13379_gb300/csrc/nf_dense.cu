@@ -255,7 +255,7 @@ __device__ __forceinline__ uint4 ld_stream_u4(const void *p) {
 // with more (3 trajectories 526 against 689 us).
 template <int NB, bool HL>
 __global__ void __launch_bounds__(DG_THREADS, NB == 1 && HL ? 4 : 2)
-gemv_kernel(const void *__restrict__ W0, const uint16_t *__restrict__ Wlo, const float *__restrict__ F, int64_t n_pad,
+gemv_kernel(const void *__restrict__ W0, const uint16_t *__restrict__ Wlo, const float *F, int64_t n_pad,
             int B, int b0, int64_t jchunk, float *__restrict__ partial) {
     constexpr int C = HL ? 8 : 4;                 // columns per load
     constexpr int UB = (HL ? 2 : 4) / (NB > 4 ? 2 : 1);  // loads per row in flight: 16 (8) x 16 bytes a lane
@@ -299,7 +299,7 @@ gemv_kernel(const void *__restrict__ W0, const uint16_t *__restrict__ Wlo, const
                 for (int v = 0; v < NB; ++v)
 #pragma unroll
                     for (int c = 0; c < C; c += 4) {
-                        const float4 f = __ldg(reinterpret_cast<const float4 *>(fp + (int64_t)v * n_pad + c));
+                        const float4 f = *reinterpret_cast<const float4 *>(fp + (int64_t)v * n_pad + c);
                         fv[v][c] = f.x, fv[v][c + 1] = f.y, fv[v][c + 2] = f.z, fv[v][c + 3] = f.w;
                     }
 #pragma unroll
@@ -352,7 +352,7 @@ constexpr size_t sym_smem_floats(int rows) {
 }
 template <int NB, bool HL>
 __global__ void __launch_bounds__(SYM_THREADS, 2)
-gemv_sym_kernel(const void *__restrict__ K, const float *__restrict__ g_all, const float *__restrict__ sc,
+gemv_sym_kernel(const void *__restrict__ K, const float *g_all, const float *__restrict__ sc,
                 int64_t n_pad, int B, int b0, int rows, float *__restrict__ partial) {
     constexpr int COLS = SB / NB;    // columns per part
     constexpr int CL = 32 / NB;      // columns per lane and part
@@ -391,7 +391,7 @@ gemv_sym_kernel(const void *__restrict__ K, const float *__restrict__ g_all, con
 #pragma unroll
             for (int v = 0; v < NB; ++v) {
                 float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (v < nv) f = __ldg(reinterpret_cast<const float4 *>(g_all + (int64_t)(b0 + v) * n_pad + node));
+                if (v < nv) f = *reinterpret_cast<const float4 *>(g_all + (int64_t)(b0 + v) * n_pad + node);
                 gj[v][c] = f.x * s4.x, gj[v][c + 1] = f.y * s4.y, gj[v][c + 2] = f.z * s4.z, gj[v][c + 3] = f.w * s4.w;
                 col[v][c] = col[v][c + 1] = col[v][c + 2] = col[v][c + 3] = 0.f;
             }

@@ -148,19 +148,19 @@ struct CInt {
 
 // Sum of base[k * stride] over k = 0 .. count - 1, added in ascending k.  The loads are
 // issued eight at a time before their adds (the order of the adds, hence the result, is that
-// of the plain loop), so each thread keeps several slot reads in flight.  base must not be
-// written by the calling kernel (read-only cache path).
-__device__ __forceinline__ float sum_slots(const float *__restrict__ base, int64_t stride, int count) {
+// of the plain loop), so each thread keeps several slot reads in flight.  Ordinary loads: the
+// kernel that wrote the slots may still have been running when the caller started (pdl_wait).
+__device__ __forceinline__ float sum_slots(const float *base, int64_t stride, int count) {
     float s = 0.f;
     int k = 0;
     for (; k + 8 <= count; k += 8) {
         float v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = __ldg(base + (int64_t)(k + j) * stride);
+        for (int j = 0; j < 8; ++j) v[j] = base[(int64_t)(k + j) * stride];
 #pragma unroll
         for (int j = 0; j < 8; ++j) s += v[j];
     }
-    for (; k < count; ++k) s += __ldg(base + (int64_t)k * stride);
+    for (; k < count; ++k) s += base[(int64_t)k * stride];
     return s;
 }
 
@@ -170,9 +170,25 @@ __device__ __forceinline__ float sum_slots(const float *__restrict__ base, int64
 // visible; at once in a normal launch), and every path of such a kernel calls it, so a kernel's
 // completion implies that of everything before it.  pdl_trigger() lets the next kernel start;
 // called after pdl_wait(), it also lets that kernel read, before its own pdl_wait(), what was
-// written up to two kernels earlier.
+// written up to two kernels earlier (with ld_l2: an SM's L1 may hold an older copy).
+// What earlier work in the stream writes is read with ordinary loads, never with __ldg or through a
+// const __restrict__ pointer: those promise that nothing writes it while the kernel runs, and the
+// kernel before still may; the compiler may also move them above the wait.  That path is for
+// what the operator's creation wrote.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Load from L2, past the SM's L1.
+__device__ __forceinline__ float ld_l2(const float *p) {
+    float v;
+    asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ long long ld_l2(const long long *p) {
+    long long v;
+    asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
 
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, bool overlap,

@@ -276,7 +276,7 @@ struct StageNode {
     int64_t node;                   // the caller's index
 };
 __device__ __forceinline__ StageNode stage_load(const StageKArgs &a, int b, int64_t i, int64_t idx) {
-    return StageNode{a.U[idx], a.us[idx], a.stage > 1 ? a.ks[idx] : 0.f, a.beta[b], a.theta[b],
+    return StageNode{ld_l2(a.U + idx), ld_l2(a.us + idx), a.stage > 1 ? ld_l2(a.ks + idx) : 0.f, a.beta[b], a.theta[b],
                      a.q ? a.q[i] : 1.f, a.perm ? (int64_t)a.perm[i] : i};
 }
 __device__ __forceinline__ void stage_update(const StageKArgs &a, const StageNode &s, long long step, int b, int64_t i,
@@ -377,7 +377,7 @@ struct FusedOut {
 };
 template <int R, int TJ, int M, int MODE>
 __global__ void __launch_bounds__(MF_THREADS, R >= 8 ? 2 : 4)
-mf_pair_packed_kernel(const float *__restrict__ xyz, const float *__restrict__ g_all, int64_t n_pad, int B, int b_base,
+mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t n_pad, int B, int b_base,
                       int64_t jchunk, float k2, float A1, float A2, float per, float *__restrict__ partial,
                       int *__restrict__ err, const __grid_constant__ FusedOut fo) {
     static_assert(M >= 0 && M <= 4, "form M: 0 general, 1 one Gaussian, 2-4 width ratio");
@@ -1109,7 +1109,7 @@ nf_status launch_prep_g(nf_operator *op, const float *u, int B, const float *bet
     return NF_OK;
 }
 
-__global__ void reduce_I_kernel(const float *__restrict__ partial, int splits, int64_t n, int64_t n_pad, int B,
+__global__ void reduce_I_kernel(const float *partial, int splits, int64_t n, int64_t n_pad, int B,
                                 const float *__restrict__ rs, const int *__restrict__ perm, float *__restrict__ I) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();
@@ -1133,7 +1133,7 @@ nf_status launch_reduce_I(nf_operator *op, int B, int splits, float *I, cudaStre
 __global__ void rk4_stage_kernel(StageKArgs a) {
     // What earlier stage kernels wrote is complete (pdl_trigger of the pair kernel in between), so
     // the state is read while the pair kernel still runs; only the partial sums wait for it.
-    const long long step = *a.step_ctr;
+    const long long step = ld_l2(a.step_ctr);
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = idx < (int64_t)a.B * a.n;
     const int b = in ? (int)(idx / a.n) : 0;
@@ -1145,7 +1145,8 @@ __global__ void rk4_stage_kernel(StageKArgs a) {
         __shared__ double time_cs[2];  // cos t, sin t of the stage
         if (threadIdx.x == 0) {
             const double cs = (a.stage == 1) ? 0.0 : (a.stage == 4 ? 1.0 : 0.5);
-            const double ts = *a.t0 + (double)step * a.dt + cs * a.dt;
+            const double t0 = __longlong_as_double(ld_l2(reinterpret_cast<const long long *>(a.t0)));
+            const double ts = t0 + (double)step * a.dt + cs * a.dt;
             sincos(ts, &time_cs[1], &time_cs[0]);
         }
         __syncthreads();

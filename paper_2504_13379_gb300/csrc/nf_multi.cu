@@ -28,7 +28,7 @@ constexpr size_t mm_smem_bytes(int nb) { return sizeof(float) * MM_TJ * (3 + (si
 
 template <int NB, int M>
 __global__ void __launch_bounds__(MM_THREADS, 2)
-mf_multi_kernel(SymNodes nd, const float *__restrict__ g, int B, int b0, int64_t jchunk, float k2, float A1, float A2,
+mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, float k2, float A1, float A2,
                 float per, float lim_tail, float lim_skip, float *__restrict__ partial) {
     static_assert(NB % 4 == 0 && NB <= 16 && M >= 0 && M <= 4, "trajectories per group, form");
     constexpr int GS = mm_stride(NB), NT = MM_TJ / kTileCols;
@@ -165,7 +165,7 @@ mf_multi_kernel(SymNodes nd, const float *__restrict__ g, int B, int b0, int64_t
             zs[k] = in ? __ldg(nd.xyz + 2 * n_pad + j) : 0.f;
             float v[NB];
 #pragma unroll
-            for (int b = 0; b < NB; ++b) v[b] = in && b < nv ? __ldg(g + (int64_t)(b0 + b) * n_pad + j) : 0.f;
+            for (int b = 0; b < NB; ++b) v[b] = in && b < nv ? g[(int64_t)(b0 + b) * n_pad + j] : 0.f;
 #pragma unroll
             for (int b = 0; b < NB; ++b) bad |= !(0.f * v[b] == 0.f);  // non-finite
 #pragma unroll

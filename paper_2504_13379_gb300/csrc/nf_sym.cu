@@ -415,7 +415,7 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
 // identically and are left out (bit-identical sums, one FMA fewer per pair).
 template <int M, int BLK, bool D2>
 __global__ void __launch_bounds__(MS_THREADS, 2)
-mf_sym_kernel(SymNodes nd, const float *__restrict__ g_all, int B, int b_base, float k2, float per, float lim_tail,
+mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float k2, float per, float lim_tail,
               float lim_skip, float *__restrict__ partial, const int *__restrict__ pairs) {
     static_assert(M >= 0 && M <= 4, "form M: 0 general, 1 one Gaussian (A2 = 0), 2-4 width ratio");
     static_assert(BLK >= 128 && BLK <= 1024 && (BLK & (BLK - 1)) == 0, "block size");
@@ -490,7 +490,7 @@ mf_sym_kernel(SymNodes nd, const float *__restrict__ g_all, int B, int b_base, f
     for (int t = 0; t < KT; ++t) {
         const int k = tid + t * MS_THREADS;
         if (k < BLK) {
-            const float gc = __ldg(g + cbase + k), gr = __ldg(g + rbase + k);
+            const float gc = g[cbase + k], gr = g[rbase + k];
             gs[k] = gc;
             rg[k] = make_float4(p[t].x, p[t].y, p[t].z, CW ? w[t].x : w[t].x * gr);
             rw[k] = w[t];
