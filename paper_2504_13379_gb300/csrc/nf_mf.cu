@@ -542,6 +542,7 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
             set_dev_error(err, DEV_TIMEOUT);
             for (int b = 0; b < 2; ++b) (void)mbar_wait_bounded(&sm.bar[b], 0), (void)mbar_wait_bounded(&sm.bar[b], 1);
         }
+        if constexpr (MODE == 1) step_done(fo.st, gridDim.x * gridDim.z);  // uncounted, it would shift later steps' count
         return;
     }
     float total = 0.f;
@@ -1162,14 +1163,15 @@ __global__ void rk4_stage_kernel(StageKArgs a) {
     step_done(a, gridDim.x);
 }
 
-// Start a new nf_rk4_advance call: clock t0 and step counter 0.
-__global__ void set_clock_kernel(double *t0_dev, long long *step_ctr, double t0) {
+// Start a new nf_rk4_advance call: clock t0, step counter 0, no block of a step counted yet.
+__global__ void set_clock_kernel(double *t0_dev, long long *step_ctr, unsigned *done_ctr, double t0) {
     *t0_dev = t0;
     *step_ctr = 0;
+    *done_ctr = 0u;
 }
 
 nf_status launch_set_clock(nf_operator *op, double t0, cudaStream_t s) {
-    set_clock_kernel<<<1, 1, 0, s>>>(op->t0_dev, op->step_ctr, t0);
+    set_clock_kernel<<<1, 1, 0, s>>>(op->t0_dev, op->step_ctr, op->done_ctr, t0);
     NF_CUDA_TRY(cudaGetLastError());
     return NF_OK;
 }
