@@ -297,6 +297,9 @@ NF_API nf_status nf_probe_pipe(int kind, int64_t iters, double *ops_per_clk_sm, 
  *   u      B x n  FP32   states (trajectory-major)
  *   beta, theta   B FP32 device arrays
  *   I      B x n  FP32   output
+ * Can be captured in a CUDA graph once a call of the same width has run (the first one
+ * allocates work arrays); the arrays that a capture names stay valid, whatever widths other
+ * calls on the operator have, until it is destroyed.
  * Errors: NF_ERR_ARG, NF_ERR_CUDA. */
 NF_API nf_status nf_nonlocal_apply(nf_operator *op, const float *u, int B, const float *beta,
                             const float *theta, float *I, void *stream);

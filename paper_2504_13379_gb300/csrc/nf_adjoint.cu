@@ -208,7 +208,7 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
     cudaStream_t s = as_stream(stream);
     const int64_t n = op->n, n_pad = op->n_pad;
     const size_t BN = (size_t)B * n;
-    NF_TRY(ensure_workspace(op, B, mf_splits(op, B)));
+    NF_TRY(ensure_workspace(op, B, mf_splits(op, B), s));
     // block-pair culling (nf_operator_mf_cull): the adjoint kernel runs over its own live
     // pairs, and each node's live W nu slots are added into slot 0 before the epilogue
     const bool cull = op->mf_cull && op->adj_pairs;

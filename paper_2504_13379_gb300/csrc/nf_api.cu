@@ -51,7 +51,29 @@ int num_sms() {
 // partial and g share one allocation, the states U, ks, us (RK4, models, adjoint) another, so a new
 // operator's first call pays for two cudaMalloc instead of five.  Each grows to the largest of its
 // parts asked for so far; sums keep their addresses when a later call of the same width adds states.
-nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state) {
+// Work arrays that a caller's stream capture names stay allocated until the operator is destroyed:
+// what a call needs does not grow with B alone (three trajectories on a small set take two g
+// buffers, or one partial slot per node block, where five take less), so a call of any other width
+// may move them, and the caller's graph still uses the old ones.
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();  // a legacy stream beside someone else's capture: not ours
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+static cudaError_t release(nf_operator *op, float **p, bool *captured) {
+    float *const old = *p;
+    *p = nullptr;
+    if (*captured) {
+        *captured = false;
+        op->retired.push_back(old);
+        return cudaSuccess;
+    }
+    return old ? cudaFree(old) : cudaSuccess;
+}
+nf_status ensure_workspace(nf_operator *op, int B, int splits, cudaStream_t s, bool state) {
     const size_t need_p = (size_t)splits * B * op->n_pad;
     const size_t need_g = (fused_fits(op, B) ? 2 : 1) * (size_t)B * op->n_pad;  // fused stages alternate
     const size_t need_s = state ? (size_t)B * op->n : 0;
@@ -60,9 +82,9 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state) {
     auto part = [](size_t have, size_t need) { return (std::max(have, need) + 63) / 64 * 64; };  // 256-byte steps
     if (sums) {
         const size_t cp = part(op->partial_cap, need_p), cg = part(op->g_cap, need_g);
-        if (op->partial) NF_CUDA_TRY(cudaFree(op->partial));
-        op->partial = op->g = nullptr;
+        op->g = nullptr;
         op->partial_cap = op->g_cap = 0;
+        NF_CUDA_TRY(release(op, &op->partial, &op->sums_captured));
         NF_CUDA_TRY(cudaMalloc(&op->partial, (cp + cg) * sizeof(float)));
         op->g = op->partial + cp;
         NF_CUDA_TRY(cudaMemset(op->g, 0, cg * sizeof(float)));  // padding columns stay zero
@@ -71,13 +93,17 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state) {
     }
     if (states) {
         const size_t cs = part(0, need_s);
-        if (op->U) NF_CUDA_TRY(cudaFree(op->U));
-        op->U = op->ks = op->us = nullptr;
+        op->ks = op->us = nullptr;
         op->state_cap = 0;
+        NF_CUDA_TRY(release(op, &op->U, &op->states_captured));
         NF_CUDA_TRY(cudaMalloc(&op->U, (op->perm ? 3 : 2) * cs * sizeof(float)));
         op->ks = op->U + cs;
         if (op->perm) op->us = op->ks + cs;
         op->state_cap = cs;
+    }
+    if (capturing(s)) {
+        op->sums_captured = true;
+        op->states_captured |= state;
     }
     return NF_OK;
 }
@@ -425,6 +451,7 @@ nf_status nf_operator_destroy(nf_operator *op) {
     cudaFree(op->rs);
     cudaFree(op->partial);  // with g
     cudaFree(op->U);        // with ks and us
+    for (float *p : op->retired) cudaFree(p);
     if (op->path == NF_GROUPED) cudaFree(op->ks);
     cudaFree(op->step_ctr);
     delete op;
@@ -456,7 +483,7 @@ nf_status nf_nonlocal_apply(nf_operator *op, const float *u, int B, const float 
         NF_TRY(tc_prep(op, u, beta, theta, false, 0, s));
         return tc_launch(op, 0, 0, I, nullptr, beta, theta, 0.0, 0, nullptr, 1, s);
     }
-    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B), false));
+    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B), s, false));
     NF_TRY(launch_prep_g(op, u, B, beta, theta, false, s));
     if (fused_fits(op, B)) return fused_apply(op, B, I, s);
     int splits = 1;
@@ -493,7 +520,7 @@ nf_status nf_rk4_advance(nf_operator *op, float *u, int B, double t0, double dt,
     }
     if (ckpt) NF_CUDA_TRY(cudaMemcpyAsync(ckpt, u, sizeof(float) * B * op->n, cudaMemcpyDeviceToDevice, s));
     if (nsteps == 0) return NF_OK;
-    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B)));
+    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B), s));
     cudaGraphExec_t exec = nullptr;
     NF_TRY(rk4_step_graph(op, u, B, dt, beta, theta, *F, ckpt, ckpt ? C : 1, &exec));
     NF_TRY(launch_prep_g(op, u, B, beta, theta, true, s));

@@ -6,6 +6,7 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 #include <cstddef>
+#include <vector>
 
 #include "../../include/nf.h"
 
@@ -277,6 +278,9 @@ struct nf_operator {
     float *ks = nullptr;         // [B][n]: RK4 slope accumulator
     size_t state_cap = 0;        // elements of U / ks
     size_t g_cap = 0;
+    // work arrays named by a caller's stream capture, and earlier ones of these (ensure_workspace)
+    bool sums_captured = false, states_captured = false;
+    std::vector<float *> retired;
     long long *step_ctr = nullptr;  // device step counter for graph replay
     unsigned *done_ctr = nullptr;   // last-block-done counter
     int *err = nullptr;             // device error flag
@@ -318,7 +322,7 @@ SplitPlan plan_splits(int64_t n_pad, int rows_per_block, int tile_cols, int resi
 void launch_validate_indices(const int32_t *idx, int64_t cnt, int64_t n, int *flag, cudaStream_t s);
 void launch_exclusive_scan(const int32_t *in, int64_t len, int32_t *out, cudaStream_t s);
 
-nf_status ensure_workspace(nf_operator *op, int B, int splits, bool state = true);
+nf_status ensure_workspace(nf_operator *op, int B, int splits, cudaStream_t s, bool state = true);
 
 // matrix-free / dense nonlocal launches (g must hold q f(U) / f(U) for B trajectories)
 nf_status mf_init_attrs();

@@ -860,7 +860,7 @@ nf_status mf_autotune(nf_operator *op, cudaStream_t s) {
     NF_CUDA_TRY(cudaEventCreate(&e1));
     float best = 1e30f;
     int best_blk = 1024;
-    NF_TRY(ensure_workspace(op, 1, (int)(op->n_pad / 512)));
+    NF_TRY(ensure_workspace(op, 1, (int)(op->n_pad / 512), s));
     NF_CUDA_TRY(cudaMemsetAsync(op->g, 0, sizeof(float) * op->n_pad, s));
     for (const int blk : {1024, 512}) {
         op->sym_blk = blk;

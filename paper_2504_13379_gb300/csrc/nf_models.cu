@@ -183,7 +183,7 @@ extern "C" nf_status nf_field_advance(nf_operator *op, const nf_model *model, in
     const bool dep = model->kind == NF_MODEL_DEPRESSION;
     const bool ab5 = integrator == NF_INTEGRATOR_AB5;
     const int64_t BN = (int64_t)B * op->n;
-    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B)));
+    NF_TRY(ensure_workspace(op, B, nonlocal_splits(op, B), cs));
     float *extra = nullptr;  // S, ksd and, with perm, ss (depression), AB5 history u (and s)
     const int64_t nextra = (dep ? (op->perm ? 3 : 2) : 0) * BN + (ab5 ? (dep ? 10 : 5) * BN : 0);
     if (nextra > 0) NF_CUDA_TRY(cudaMallocAsync(&extra, sizeof(float) * nextra, cs));
