@@ -87,7 +87,13 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits, cudaStream_t s, b
         NF_CUDA_TRY(release(op, &op->partial, &op->sums_captured));
         NF_CUDA_TRY(cudaMalloc(&op->partial, (cp + cg) * sizeof(float)));
         op->g = op->partial + cp;
-        NF_CUDA_TRY(cudaMemset(op->g, 0, cg * sizeof(float)));  // padding columns stay zero
+        // Padding columns stay zero.  Cleared on the stream that uses them: on the default stream the
+        // clearing could run after the first kernels of a non-blocking one.  (A capture in relaxed
+        // mode gets this far; the clearing is then done now, not in the graph.)
+        if (capturing(s))
+            NF_CUDA_TRY(cudaMemset(op->g, 0, cg * sizeof(float)));
+        else
+            NF_CUDA_TRY(cudaMemsetAsync(op->g, 0, cg * sizeof(float), s));
         op->partial_cap = cp;
         op->g_cap = cg;
     }
