@@ -140,12 +140,13 @@ adj_sym_kernel(SymNodes nd, const float *nu_all, const float *g_all, int B, int 
     for (int ps = warp; ps < NPASS; ps += AS_WARPS) {
         const int r0 = ps * R, grp = r0 / kPassRows;
         if (rbase + r0 >= nd.n) break;  // padding: no row to write, nu = g = 0 in every other sum
-        const float4 c = pc[grp];
+        const float4 c = pc[grp], e = pe[grp];
         float d2 = 3.4e38f;
-        if (lane < ntile) d2 = box_d2(c, pe[grp], tcs[lane], tes[lane], per, iper);
+        if (lane < ntile) d2 = box_d2(c, e, tcs[lane], tes[lane], per, iper);
         const unsigned live_t = __ballot_sync(0xffffffffu, lane < ntile && d2 <= lim_skip);
-        // periodic distances take plain differences, reduced pair by pair
-        const bool local = c.w == 1.f && !(per > 0.f);  // warp-uniform
+        // periodic distances take plain differences, reduced pair by pair; so do rows that the forward
+        // sums expand for the first Gaussian alone (A2 = 0) but that lie too far apart for the second
+        const bool local = c.w == 1.f && !(per > 0.f) && (M > 0 || k2 * e.w <= kSymLocalSpread);  // warp-uniform
         const unsigned full_t = local ? live_t & __ballot_sync(0xffffffffu, d2 <= lim_tail) : live_t;
         const unsigned tail_t = live_t & ~full_t;
         // per row, over the lane's columns j (e1, e2 without the row factors):
@@ -158,7 +159,7 @@ adj_sym_kernel(SymNodes nd, const float *nu_all, const float *g_all, int B, int 
             float4 p = rg[r0 + r];
             float2 w = rw[r0 + r];
             const float nui = rnu[r0 + r], gi = diag ? 0.f : rgv[r0 + r];
-            if (per > 0.f) {
+            if (!local) {
                 p.x = __ldg(nd.xyz + rbase + r0 + r);
                 p.y = __ldg(nd.xyz + n_pad + rbase + r0 + r);
                 p.z = __ldg(nd.xyz + 2 * n_pad + rbase + r0 + r);
@@ -273,7 +274,7 @@ adj_sym_kernel(SymNodes nd, const float *nu_all, const float *g_all, int B, int 
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             // the row factors 2^(-n_i) of e1 and e2 (n_i = 0 outside the expanded form)
-            const float ni = per > 0.f ? 0.f : rg[r0 + r].w;
+            const float ni = local ? rg[r0 + r].w : 0.f;
             const float f1 = exp2f(M > 0 ? -(float)M * ni : -ni), f2 = exp2f(M > 0 ? -ni : -k2 * ni);
             if constexpr (CW) {
                 const float P1s = f2_fold(b1[r]), P2s = f2_fold(b2[r]);

@@ -346,7 +346,7 @@ struct MfPackedSmem {
 // operations shared by the warp's R rows; per pair the exponent argument is then a chain
 // of 3 FMAs instead of 3 SUB + MUL + 2 FMA.  FP32 rounding of s_ij is relative to
 // n_i + n_j + 2 |x_i - c||x_j - c|, so the form is used only when every row of the warp has
-// n_i <= kMfLocalSpread (scaled units, i.e. |x_i - c| <= s1 / sqrt(log2 e)); for pairs
+// n_i <= kMfLocalSpread (in units of the narrower Gaussian evaluated: |x_i - c| <= s / sqrt(log2 e)); for pairs
 // that carry weight this keeps the error at a few ulps of r^2, the same order as the
 // rounding of the stored coordinates.  Warps whose rows are spread out use the difference
 // form.  The choice is warp-uniform and fixed per launch shape, so results stay
@@ -445,9 +445,10 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
         const float dx = xr[r] - cx, dy = yr[r] - cy, dz = zr[r] - cz;
         spread = fmaxf(spread, dx * dx + dy * dy + dz * dz);
     }
-    // warp-uniform, the threshold in the stored units; periodic distances take the difference
-    // form (nearest images per pair)
-    const bool local = spread <= (M >= 2 ? kMfLocalSpread * k2 : kMfLocalSpread) && !(per > 0.f);
+    // warp-uniform, the threshold in the stored units, for the narrower Gaussian evaluated; periodic
+    // distances take the difference form (nearest images per pair)
+    const float most = M >= 2 ? kMfLocalSpread * k2 : (M == 0 ? kMfLocalSpread / fmaxf(1.f, k2) : kMfLocalSpread);
+    const bool local = spread <= most && !(per > 0.f);
     // local: xi, yi, zi hold -2 (x_i - c); otherwise x_i itself (both halves of the pair)
     const float lsc = -2.f;
     u64 xi[R], yi[R], zi[R], a1[R], a2[R];

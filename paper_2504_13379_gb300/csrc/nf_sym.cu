@@ -42,15 +42,6 @@
 
 namespace nfi {
 
-// The expanded form's threshold: rows within 2 s1 / sqrt(log2 e) of their centre.  The
-// rounding of r^2 = n_i + s_ij for the pairs that carry weight stays of order eps * n_i
-// (below 3e-7 relative in the exponential at n_i = 4); the expanded form saves three of the
-// difference form's six exponent operations per pair.  Measured on GB300 against a threshold
-// of 1: the same error against the FP64 oracle (1.4e-7 relative L2 on the precision torus,
-// 9.3e-7 on the periodic square), 2.37 vs 2.63 ms on the periodic square at n = 131,072,
-// 0.157 vs 0.175 ms on the 20,000-node sphere.
-constexpr float kSymLocalSpread = 4.0f;
-
 constexpr int MS_THREADS = 256;
 constexpr int MS_WARPS = MS_THREADS / 32;
 // shared memory (4-byte words): columns x, y, z, g (4 BLK); row operands, factors and weights
@@ -184,7 +175,9 @@ __global__ void sym_static_kernel(const float *__restrict__ xyz, int64_t n_pad, 
         }
     }
     pc[ps] = make_float4(c.x, c.y, c.z, (float)form);
-    pe[ps] = bx.half(c);
+    float4 he = bx.half(c);
+    he.w = spread;
+    pe[ps] = he;
     const bool centred = form >= 2;
     for (int r = 0; r < kPassRows; ++r) {
         const int64_t k = r0 + r;
@@ -393,9 +386,12 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     }
     pack_sorted_kernel<<<(unsigned)ceil_div(n_pad, 256), 256, 0, s>>>(x, q, keys, n, n_pad, mf_unit(op), op->x4,
                                                                      op->xyz, op->q, op->perm);
-    // the threshold of the expanded form in the stored units
+    // the threshold of the expanded form in the stored units, for the narrower of the Gaussians that
+    // the forward sums evaluate
     const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
-    const float spread = op->form >= 2 ? kSymLocalSpread * k2 : kSymLocalSpread;
+    const float spread = op->form >= 2   ? kSymLocalSpread * k2
+                         : op->form == 0 ? kSymLocalSpread / std::max(1.f, k2)
+                                         : kSymLocalSpread;
     sym_static_kernel<<<(unsigned)ceil_div(np, 128), 128, 0, s>>>(op->xyz, n_pad, op->form, k2, k.A1, k.A2,
                                                                  mf_period(op), spread, op->rg, op->rw, op->pc, op->pe);
     sym_tiles_kernel<<<(unsigned)ceil_div(32 * nt, 128), 128, 0, s>>>(op->xyz, n_pad, op->tc, op->te);
