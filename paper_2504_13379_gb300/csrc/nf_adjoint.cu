@@ -255,8 +255,6 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
         for (int j = 0; j < cnt; ++j) {
             for (int stage = 1; stage <= 4; ++stage) {
                 if (stage == 4 && j + 1 == cnt) break;  // its sum only leads to the next segment's state
-                int splits = 1;
-                NF_TRY(launch_mf_pair(op, B, ss, &splits));
                 StageParams p{};
                 p.u = nullptr;  // the state advances inside the operator only
                 p.beta = beta;
@@ -266,9 +264,14 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 p.stage = stage;
                 p.ckpt = nullptr;
                 p.C = 1;
-                p.splits = splits;
                 p.overlap = true;
                 p.stage_out = st + ((size_t)j * 4 + stage) * BN;
+                // the forward run's kernels: the stage inputs are its own to the last bit
+                if (fused_fits(op, B) && F.kind == NF_FORCE_NONE) {
+                    NF_TRY(fused_stage(op, B, p, ss));
+                    continue;
+                }
+                NF_TRY(launch_mf_pair(op, B, ss, &p.splits));
                 NF_TRY(launch_stage(op, B, p, ss));
             }
         }
