@@ -254,7 +254,6 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
         NF_CUDA_TRY(cudaMemcpyAsync(st, op->U, sizeof(float) * BN, cudaMemcpyDeviceToDevice, ss));
         for (int j = 0; j < cnt; ++j) {
             for (int stage = 1; stage <= 4; ++stage) {
-                if (stage == 4 && j + 1 == cnt) break;  // its sum only leads to the next segment's state
                 StageParams p{};
                 p.u = nullptr;  // the state advances inside the operator only
                 p.beta = beta;
@@ -265,7 +264,8 @@ extern "C" nf_status nf_adjoint(nf_operator *op, const float *ckpt, int C, int B
                 p.ckpt = nullptr;
                 p.C = 1;
                 p.overlap = true;
-                p.stage_out = st + ((size_t)j * 4 + stage) * BN;
+                // the segment's last state is the next checkpoint: computed for its check alone
+                if (stage < 4 || j + 1 < cnt) p.stage_out = st + ((size_t)j * 4 + stage) * BN;
                 // the forward run's kernels: the stage inputs are its own to the last bit
                 if (fused_fits(op, B) && F.kind == NF_FORCE_NONE) {
                     NF_TRY(fused_stage(op, B, p, ss));
