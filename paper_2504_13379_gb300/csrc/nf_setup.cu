@@ -413,8 +413,15 @@ static nf_status build_stencils(const double *nodes, int64_t n, int dim, const i
     // FP32 offsets are off by up to 2^-24 of the grid's extent each, per coordinate and node
     const double rel = 4.0 * 5.97e-8 * (double)std::max(gr.G[0], std::max(gr.G[1], gr.G[2]));
     const float margin = (float)((1.0 + rel) * (1.0 + rel) * (1.0 + 1e-5));
-    knn_warp_kernel<<<(unsigned)ceil_div(m, KNN_WARPS), 32 * KNN_WARPS, 0, s>>>(
-        nodes, dim, m, k, gr, rho0, margin, start, sorted, sx, qc, qcell, stencils, left);
+    // Coordinates so large or small that squared FP32 offsets leave FP32's normal range: the rejection
+    // would decide wrongly, so every query goes to the thread kernel, which works in FP64 alone.
+    if (gr.h > 1e-12 && ext < 1e18) {
+        knn_warp_kernel<<<(unsigned)ceil_div(m, KNN_WARPS), 32 * KNN_WARPS, 0, s>>>(
+            nodes, dim, m, k, gr, rho0, margin, start, sorted, sx, qc, qcell, stencils, left);
+    } else {
+        NF_CUDA_TRY(cudaMemsetAsync(stencils, 0xff, sizeof(int32_t) * m * k, s));
+        NF_CUDA_TRY(cudaMemsetAsync(left, 1, sizeof(int), s));
+    }
     knn_query_kernel<<<(unsigned)ceil_div(m, 128), 128, 0, s>>>(nodes, n, dim, m, k, gr, start, sorted, qc, qcell,
                                                                 stencils, left);
     NF_CUDA_TRY(cudaGetLastError());
