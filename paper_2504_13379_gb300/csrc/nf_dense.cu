@@ -647,9 +647,13 @@ static SplitPlan gemm_plan(const nf_operator *op, int B) {
     return p;
 }
 
-// Small planes give the GEMM too few tiles (12 CTAs at n = 1,500: 90 us per sum of 64 trajectories).
+// Planes of up to 2,048 padded nodes give the GEMM few tiles: 94 to 140 us per sum for any number of
+// trajectories, while a pass of 8 over the plane, which stays in L2, takes 6.  Per sum at
+// n = 2,000, passes / GEMM: 64 trajectories 55 / 96 us, 128 105 / 136, 192 154 / 137, 256 203 / 138,
+// 512 394 / 142 (n = 700: 52 / 96, 98 / 136, 146 / 136, 192 / 136, 377 / 136).
+constexpr int kGemmMinBSmall = 169;
 static bool use_gemm(const nf_operator *op, int B) {
-    return op->path == NF_DENSE_FP32 && B >= kGemmMinB && op->n_pad >= 3072;
+    return op->path == NF_DENSE_FP32 && B >= (op->n_pad > 2048 ? kGemmMinB : kGemmMinBSmall);
 }
 
 template <int NB>
