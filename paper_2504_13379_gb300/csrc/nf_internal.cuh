@@ -253,6 +253,7 @@ struct nf_operator {
     int adj_blk = 0;         // node block of the adjoint pair kernel (0: not yet timed; 1024 or 512)
     int mf_sched = 0;        // NF_MF_AUTO / NF_MF_SYMMETRIC / NF_MF_PACKED
     int sym_blk = 1024;      // node block of the symmetric kernel (1024, or 512 when autotuned faster)
+    int auto_blk = 0;        // its small block (256, 128) where the node count alone chooses it, else 0
     int planar = 0;          // every node has the same z: the symmetric kernel drops the z terms
     // block-pair culling of the symmetric kernel (opt-in, nf_operator_mf_cull)
     int mf_cull = 0;

@@ -841,7 +841,7 @@ nf_status mf_autotune(nf_operator *op, cudaStream_t s) {
     op->mf_variant = default_variant(op->n_pad);
     if (!sym_layout_fits(op)) return NF_OK;  // packed by default
     if (3 * sym_pairs_1024(op) < 2 * (int64_t)num_sms()) {
-        op->sym_blk = op->n > kFusedMaxN ? 256 : 128;  // 128: only when the schedule asks for symmetric
+        op->sym_blk = op->auto_blk = op->n > kFusedMaxN ? 256 : 128;  // 128: only when the schedule asks for symmetric
         return NF_OK;
     }
     // 512-node blocks only where 1,024-node pairs fill fewer than four waves of two CTAs per
