@@ -226,6 +226,12 @@ __device__ __forceinline__ float bf16_bits_to_float(uint32_t h) { return __uint_
 // columns contribute nothing and every tile is full.
 constexpr int64_t kNodePad = 1024;
 
+// Units of the exact node data (nf_operator::xyz2): stored coordinates per unit of the caller's (a power
+// of two), exponent per squared stored unit, the second exponent's ratio to it, the period.
+struct ExactUnits {
+    float unit, uu, k2, per;
+};
+
 struct nf_graph_cache;
 struct nf_group_state;
 
@@ -248,6 +254,13 @@ struct nf_operator {
     float4 *rg = nullptr;    // node data of the symmetric kernels (SymNodes), one allocation from rg on
     float2 *rw = nullptr;
     float4 *pc = nullptr, *pe = nullptr, *tc = nullptr, *te = nullptr;
+    // The same node data over the caller's coordinates times a power of two, that is over exact
+    // ones, for the packed, 256-node-block and multi-trajectory kernels (ExactUnits).
+    float *xyz2 = nullptr;
+    float4 *rg2 = nullptr;
+    float2 *rw2 = nullptr;
+    float4 *pc2 = nullptr, *pe2 = nullptr, *tc2 = nullptr, *te2 = nullptr;
+    ExactUnits eu{};
     int mf_variant = -1;     // launch shape of the packed pair kernel
     int adj_r = 0;           // rows per warp of the adjoint pair kernel (0: not yet timed; 4 or 8)
     int adj_blk = 0;         // node block of the adjoint pair kernel (0: not yet timed; 1024 or 512)

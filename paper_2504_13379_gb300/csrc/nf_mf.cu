@@ -328,8 +328,8 @@ __device__ __forceinline__ void step_done(const StageKArgs &a, unsigned blocks) 
 // the FMA pipe).  Column tiles are staged as structure-of-arrays (x, y, z, g), so a
 // lane reads two adjacent columns with one 8-byte load; each row's coordinates are held
 // duplicated in a 64-bit register pair.  Difference form, per two pairs: 3 SUB2, MUL2 +
-// 2 FMA2 (r^2), MUL2 (second exponent), 4 MUFU.EX2, 2 FMA2 -- the rounding of the scalar
-// kernel.  Expanded form (below): 3 FMA2, MUL2, 4 MUFU.EX2, 2 FMA2, plus 6 per column pair
+// 2 FMA2 (r^2), MUL2 (exponent), MUL2 (second exponent), 4 MUFU.EX2, 2 FMA2 -- the rounding of the
+// scalar kernel.  Expanded form (below): 3 FMA2, MUL2, 4 MUFU.EX2, 2 FMA2, plus 6 per column pair
 // shared by the warp's rows, which leaves the SFU (2 exponentials per pair) as the bound.
 template <int TJ>
 struct MfPackedSmem {
@@ -344,22 +344,25 @@ struct MfPackedSmem {
 // and accumulates 2^(-s_ij) and 2^(-k2 s_ij); the row factors 2^(-n_i), 2^(-k2 n_i) are
 // applied once at the end.  Per column pair the centred coordinates and n_j cost 6 lane
 // operations shared by the warp's R rows; per pair the exponent argument is then a chain
-// of 3 FMAs instead of 3 SUB + MUL + 2 FMA.  FP32 rounding of s_ij is relative to
+// of 3 FMAs instead of 3 SUB + 2 MUL + 2 FMA.  FP32 rounding of s_ij is relative to
 // n_i + n_j + 2 |x_i - c||x_j - c|, so the form is used only when every row of the warp has
-// n_i <= kMfLocalSpread (in units of the narrower Gaussian evaluated: |x_i - c| <= s / sqrt(log2 e)); for pairs
-// that carry weight this keeps the error at a few ulps of r^2, the same order as the
-// rounding of the stored coordinates.  Warps whose rows are spread out use the difference
-// form.  The choice is warp-uniform and fixed per launch shape, so results stay
-// deterministic.
+// n_i <= kMfLocalSpread as an exponent of the narrower Gaussian evaluated (|x_i - c| <= s / 2.4, s its
+// width).  Warps whose rows are spread out use the difference form.  The choice is warp-uniform
+// and fixed per launch shape, so results stay deterministic.  The threshold trades rounding for
+// time at 2,000 to 3,000 nodes: over 56 kernels and node sets of 500 to 3,001 nodes the relative L2 error
+// against FP64 has a geometric mean of 0.78e-7 with 0.25 as with 0.5, and at worst 2.6e-7 against 3.5e-7
+// (a lattice on which the two Gaussians nearly cancel); 0.0625 takes 5 to 8 % longer.  Coordinates
+// rounded to exponent units and exp2f's row factors gave 1.32e-7, at worst 7.4e-7.
 //
 // Integer width ratio.  When m = s2^2 / s1^2 is a small integer (M = 2, 3, 4; the paper's
-// lateral-inhibition kernels have sigma_i = 2 sigma_e, i.e. m = 4), the expanded form works
-// in units of s2 and takes e2 = 2^(-s'_ij) from the SFU and e1 = e2^M by squaring on the FMA pipe: one exponential per pair
-// instead of two.  The relative error of e1 grows to about M times that of ex2.approx
-// (a few 1e-7).  M = 0 is the general form.
-constexpr float kMfLocalSpread = 1.0f;
+// lateral-inhibition kernels have sigma_i = 2 sigma_e, i.e. m = 4), the expanded form takes
+// e2 = 2^(-s_ij), in units of s2, from the SFU and e1 = e2^M by squaring on the FMA pipe: one
+// exponential per pair instead of two.  The relative error of e1 grows to about M times that of
+// ex2.approx (a few 1e-7).  M = 0 is the general form.
+constexpr float kMfLocalSpread = 0.25f;
 
-// xyz: coordinates in exponent units as structure of arrays [x(n_pad) | y(n_pad) | z(n_pad)];
+// xyz: the exact set's coordinates (times a power of two; the exponent of a pair is uu r^2) as
+// structure of arrays [x(n_pad) | y(n_pad) | z(n_pad)];
 // g_all: B x n_pad firing rates (times q); both in Hilbert order, like the partial sums.
 //
 // MODE 0 writes partial sums.  Small node sets (MODE 1, 2: one column split, so a warp holds the
@@ -378,7 +381,7 @@ struct FusedOut {
 template <int R, int TJ, int M, int MODE>
 __global__ void __launch_bounds__(MF_THREADS, R >= 8 ? 2 : 4)
 mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t n_pad, int B, int b_base,
-                      int64_t jchunk, float k2, float A1, float A2, float per, float *__restrict__ partial,
+                      int64_t jchunk, float uu, float k2, float A1, float A2, float per, float *__restrict__ partial,
                       int *__restrict__ err, const __grid_constant__ FusedOut fo) {
     static_assert(M >= 0 && M <= 4, "form M: 0 general, 1 one Gaussian, 2-4 width ratio");
     __shared__ __align__(128) MfPackedSmem<TJ> sm;
@@ -411,6 +414,60 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
         if (ntiles > 0) issue_xyz(0);
         if (ntiles > 1) issue_xyz(1);
     }
+    // the warp's rows (all lanes hold the same values) and the centre of their bounding box
+    float xr[R], yr[R], zr[R];
+    float lox = 3.4e38f, loy = 3.4e38f, loz = 3.4e38f, hix = -3.4e38f, hiy = -3.4e38f, hiz = -3.4e38f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        xr[r] = X[slot0 + r];
+        yr[r] = Y[slot0 + r];
+        zr[r] = Z[slot0 + r];
+        lox = fminf(lox, xr[r]), hix = fmaxf(hix, xr[r]);
+        loy = fminf(loy, yr[r]), hiy = fmaxf(hiy, yr[r]);
+        loz = fminf(loz, zr[r]), hiz = fmaxf(hiz, zr[r]);
+    }
+    const float cx = 0.5f * (lox + hix), cy = 0.5f * (loy + hiy), cz = 0.5f * (loz + hiz);
+    // Expanded form: coordinates centred and scaled in one FMA, w x - w c with w = sqrt(uu): the same one
+    // rounding of the difference as in x - c, and no multiplication by uu left in the loop.
+    const float w = sqrtf(uu), ncx = -(w * cx), ncy = -(w * cy), ncz = -(w * cz);
+    float spread = 0.f;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float dx = fmaf(w, xr[r], ncx), dy = fmaf(w, yr[r], ncy), dz = fmaf(w, zr[r], ncz);
+        spread = fmaxf(spread, dx * dx + dy * dy + dz * dz);
+    }
+    // warp-uniform, the threshold as an exponent, for the narrower Gaussian evaluated; periodic
+    // distances take the difference form (nearest images per pair)
+    const float most = M >= 2 ? kMfLocalSpread * k2 : (M == 0 ? kMfLocalSpread / fmaxf(1.f, k2) : kMfLocalSpread);
+    const bool local = spread <= most && !(per > 0.f);
+    // local: xi, yi, zi hold -2 w (x_i - c); otherwise x_i itself (both halves of the pair).
+    // M >= 2: one pair weight e2 + c_i e1, c_i = -(A1 f1) / (A2 f2) with the row factors, and one sum: the
+    // difference of the two Gaussians' sums magnifies the rounding of either (see nf_sym.cu)
+    constexpr bool CW = M >= 2;
+    u64 xi[R], yi[R], zi[R], h1[CW ? R : 1], a1[R], a2[CW ? 1 : R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const float x = local ? -2.f * fmaf(w, xr[r], ncx) : xr[r];
+        const float y = local ? -2.f * fmaf(w, yr[r], ncy) : yr[r];
+        const float z = local ? -2.f * fmaf(w, zr[r], ncz) : zr[r];
+        xi[r] = f2_pack(x, x);
+        yi[r] = f2_pack(y, y);
+        zi[r] = f2_pack(z, z);
+        a1[r] = 0ull;
+        if constexpr (CW) {
+            const float ni = local ? 0.25f * (x * x + y * y + z * z) : 0.f;
+            h1[r] = f2_dup(scale_pow2(-(A1 / A2), -(float)(M - 1) * ni, local ? kEx2Low : 0.f));
+        } else {
+            a2[r] = 0ull;
+        }
+    }
+    // with a = uu r^2 the exponent of a pair: M < 2: e1 = 2^(-a), e2 = 2^(-k2 a) with
+    // k2 = s1^2 / s2^2; M >= 2: e2 = 2^(-a), e1 = 2^(-M a)
+    const u64 uup = f2_dup(uu);
+    const u64 nk2 = M >= 2 ? f2_dup(-(float)M) : f2_dup(-k2);
+    const u64 wp = f2_dup(w), cxp = f2_dup(ncx), cyp = f2_dup(ncy), czp = f2_dup(ncz);
+    const float iper = per > 0.f ? 1.f / per : 0.f;
+    const u64 ipp = f2_pack(iper, iper), npp = f2_pack(-per, -per), mgp = f2_pack(kRintMagic, kRintMagic);
     // MODE 1: lane r < R carries row r's state
     long long step = 0;
     StageNode sn{};
@@ -426,49 +483,6 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
         if (ntiles > 0) issue_g(0);
         if (ntiles > 1) issue_g(1);
     }
-    // the warp's rows (all lanes hold the same values) and the centre of their bounding box
-    float xr[R], yr[R], zr[R];
-    float lox = 3.4e38f, loy = 3.4e38f, loz = 3.4e38f, hix = -3.4e38f, hiy = -3.4e38f, hiz = -3.4e38f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        xr[r] = X[slot0 + r];
-        yr[r] = Y[slot0 + r];
-        zr[r] = Z[slot0 + r];
-        lox = fminf(lox, xr[r]), hix = fmaxf(hix, xr[r]);
-        loy = fminf(loy, yr[r]), hiy = fmaxf(hiy, yr[r]);
-        loz = fminf(loz, zr[r]), hiz = fmaxf(hiz, zr[r]);
-    }
-    const float cx = 0.5f * (lox + hix), cy = 0.5f * (loy + hiy), cz = 0.5f * (loz + hiz);
-    float spread = 0.f;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const float dx = xr[r] - cx, dy = yr[r] - cy, dz = zr[r] - cz;
-        spread = fmaxf(spread, dx * dx + dy * dy + dz * dz);
-    }
-    // warp-uniform, the threshold in the stored units, for the narrower Gaussian evaluated; periodic
-    // distances take the difference form (nearest images per pair)
-    const float most = M >= 2 ? kMfLocalSpread * k2 : (M == 0 ? kMfLocalSpread / fmaxf(1.f, k2) : kMfLocalSpread);
-    const bool local = spread <= most && !(per > 0.f);
-    // local: xi, yi, zi hold -2 (x_i - c); otherwise x_i itself (both halves of the pair)
-    const float lsc = -2.f;
-    u64 xi[R], yi[R], zi[R], a1[R], a2[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const float x = local ? lsc * (xr[r] - cx) : xr[r];
-        const float y = local ? lsc * (yr[r] - cy) : yr[r];
-        const float z = local ? lsc * (zr[r] - cz) : zr[r];
-        xi[r] = f2_pack(x, x);
-        yi[r] = f2_pack(y, y);
-        zi[r] = f2_pack(z, z);
-        a1[r] = 0ull;
-        a2[r] = 0ull;
-    }
-    // coordinates arrive in exponent units: M < 2: e1 = 2^(-r2), e2 = 2^(-k2 r2) with
-    // k2 = s1^2 / s2^2; M >= 2: e2 = 2^(-r2), e1 = 2^(-M r2)
-    const u64 nk2 = M >= 2 ? f2_dup(-(float)M) : f2_dup(-k2);
-    const u64 cxp = f2_dup(cx), cyp = f2_dup(cy), czp = f2_dup(cz);
-    const float iper = per > 0.f ? 1.f / per : 0.f;
-    const u64 ipp = f2_pack(iper, iper), npp = f2_pack(-per, -per), mgp = f2_pack(kRintMagic, kRintMagic);
     bool timed_out = false;
     for (int t = 0; t < ntiles; ++t) {
         const int buf = t & 1;
@@ -488,7 +502,7 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
         if (local) {
 #pragma unroll 2
             for (int jp = lane; jp < TJ / 2; jp += 32) {
-                const u64 xt = f2_sub(xs[jp], cxp), yt = f2_sub(ys[jp], cyp), zt = f2_sub(zs[jp], czp);
+                const u64 xt = f2_fma(xs[jp], wp, cxp), yt = f2_fma(ys[jp], wp, cyp), zt = f2_fma(zs[jp], wp, czp);
                 const u64 nj = f2_fma(zt, zt, f2_fma(yt, yt, f2_mul(xt, xt)));
                 const u64 gj = gs[jp];
 #pragma unroll
@@ -497,10 +511,9 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
                     float s0, s1v;
                     f2_unpack(sij, s0, s1v);
                     const u64 e = f2_pack(ex2_sfu(-s0), ex2_sfu(-s1v));
-                    if constexpr (M >= 2) {
+                    if constexpr (CW) {
                         const u64 sq = f2_mul(e, e);
-                        a1[r] = f2_fma(M == 2 ? sq : (M == 3 ? f2_mul(sq, e) : f2_mul(sq, sq)), gj, a1[r]);
-                        a2[r] = f2_fma(e, gj, a2[r]);
+                        a1[r] = f2_fma(f2_fma(M == 2 ? sq : (M == 3 ? f2_mul(sq, e) : f2_mul(sq, sq)), h1[r], e), gj, a1[r]);
                     } else {
                         a1[r] = f2_fma(e, gj, a1[r]);
                         if constexpr (M == 0) a2[r] = f2_fma(f2_ex2(f2_mul(sij, nk2)), gj, a2[r]);
@@ -521,14 +534,17 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
                         dx = f2_wrap(dx, ipp, npp, mgp);
                         dy = f2_wrap(dy, ipp, npp, mgp);
                     }
-                    const u64 r2s = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+                    const u64 r2s = f2_mul(f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))), uup);
                     float s0, s1v;
                     f2_unpack(r2s, s0, s1v);
                     // 2^(-r2s): the narrow Gaussian, or for M >= 2 the wide one
                     const u64 e = f2_pack(ex2_sfu(-s0), ex2_sfu(-s1v));
-                    (M >= 2 ? a2[r] : a1[r]) = f2_fma(e, gj, M >= 2 ? a2[r] : a1[r]);
-                    if constexpr (M >= 2) a1[r] = f2_fma(f2_ex2(f2_mul(r2s, nk2)), gj, a1[r]);
-                    if constexpr (M == 0) a2[r] = f2_fma(f2_ex2(f2_mul(r2s, nk2)), gj, a2[r]);
+                    if constexpr (CW) {
+                        a1[r] = f2_fma(f2_fma(f2_ex2(f2_mul(r2s, nk2)), h1[r], e), gj, a1[r]);
+                    } else {
+                        a1[r] = f2_fma(e, gj, a1[r]);
+                        if constexpr (M == 0) a2[r] = f2_fma(f2_ex2(f2_mul(r2s, nk2)), gj, a2[r]);
+                    }
                 }
             }
             };
@@ -549,18 +565,17 @@ mf_pair_packed_kernel(const float *__restrict__ xyz, const float *g_all, int64_t
     float total = 0.f;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        float p0, p1, q0, q1;
-        f2_unpack(a1[r], p0, p1);
-        f2_unpack(a2[r], q0, q1);
-        float s1f = A1 * (p0 + p1), s2f = A2 * (q0 + q1);
+        // first sum, with the factor of its Gaussian (M >= 2: of the wide one), then the second
+        float s1f = (CW ? -A2 : A1) * f2_fold(a1[r]), s2f = 0.f;
+        if constexpr (M == 0) s2f = A2 * f2_fold(a2[r]);
         if (local) {  // n_i from the same rounded centred coordinates the loop used
             float mx, my, mz, unused;
             f2_unpack(xi[r], mx, unused);
             f2_unpack(yi[r], my, unused);
             f2_unpack(zi[r], mz, unused);
             const float ni = 0.25f * (mx * mx + my * my + mz * mz);  // in units of s2 when M >= 2
-            s1f *= exp2f(M >= 2 ? -(float)M * ni : -ni);
-            s2f *= exp2f(M >= 2 ? -ni : -k2 * ni);
+            s1f = scale_pow2(s1f, -ni, kEx2Low);
+            if constexpr (M == 0) s2f = scale_pow2(s2f, -k2 * ni, kEx2Low);
         }
         const float v = warp_sum(s1f - s2f);
         if constexpr (MODE == 0) {
@@ -690,10 +705,10 @@ static int variant_resident(int v) {
 template <int R, int TJ>
 static void launch_packed(nf_operator *op, int B, int b_base, int groups, const SplitPlan &pl, cudaStream_t s) {
     const nf_kernel &k = op->kp;
-    const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
+    const ExactUnits &eu = op->eu;
     dim3 grid((unsigned)pl.row_blocks, (unsigned)pl.splits, (unsigned)groups);
 #define NF_PACKED_ARGS \
-    op->xyz, op->g, op->n_pad, B, b_base, pl.jchunk, k2, k.A1, k.A2, mf_period(op), op->partial, op->err, FusedOut{}
+    op->xyz2, op->g, op->n_pad, B, b_base, pl.jchunk, eu.uu, eu.k2, k.A1, k.A2, eu.per, op->partial, op->err, FusedOut{}
     switch (op->form) {
         case 1: mf_pair_packed_kernel<R, TJ, 1, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
         case 2: mf_pair_packed_kernel<R, TJ, 2, 0><<<grid, MF_THREADS, 0, s>>>(NF_PACKED_ARGS); break;
@@ -740,12 +755,12 @@ template <int MODE>
 static cudaError_t launch_fused(nf_operator *op, int B, const float *g, const FusedOut &fo, bool overlap, cudaStream_t s) {
     constexpr int R = kFusedRows, TJ = kFusedTile;
     const nf_kernel &k = op->kp;
-    const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
+    const ExactUnits &eu = op->eu;
     // row blocks with a real node only; every column tile
     const dim3 grid((unsigned)ceil_div(op->n, MF_WARPS * R), 1, (unsigned)B);
     auto go = [&](auto kernel) {
-        return launch_dependent(kernel, grid, MF_THREADS, 0, s, overlap, op->xyz, g, op->n_pad, B, 0, op->n_pad, k2,
-                                k.A1, k.A2, mf_period(op), (float *)nullptr, op->err, fo);
+        return launch_dependent(kernel, grid, MF_THREADS, 0, s, overlap, op->xyz2, g, op->n_pad, B, 0, op->n_pad,
+                                eu.uu, eu.k2, k.A1, k.A2, eu.per, (float *)nullptr, op->err, fo);
     };
     switch (op->form) {
         case 1: return go(mf_pair_packed_kernel<R, TJ, 1, MODE>);

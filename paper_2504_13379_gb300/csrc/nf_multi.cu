@@ -21,6 +21,13 @@ namespace nfi {
 
 constexpr int MM_THREADS = 256, MM_WARPS = MM_THREADS / 32, MM_R = 4, MM_TJ = 512;
 constexpr int MM_ROWS = MM_WARPS * MM_R;
+// Threshold of the expanded form, half of the symmetric kernels'.  Geometric mean over 32 kernels and node
+// sets (n = 500 to 15,000) of the relative L2 error against FP64: 0.78e-7 (0.80e-7 with their threshold,
+// which is up to 4 % faster at 8,000 nodes; 0.77e-7 with half of this one, up to 4 % slower).  The
+// scalar kernel that served every width before, on plain differences of the caller's
+// coordinates, has 0.76e-7; with coordinates rounded to exponent units and exp2f's row factors
+// this kernel had 1.20e-7.
+constexpr float kMultiSpread = 2.0f;
 // floats per column of the transposed g tile: strides of 4, 12 and 20 words spread eight adjacent
 // columns' 16-byte reads over all banks
 constexpr int mm_stride(int nb) { return nb == 8 ? 12 : (nb == 16 ? 20 : nb); }
@@ -28,8 +35,8 @@ constexpr size_t mm_smem_bytes(int nb) { return sizeof(float) * MM_TJ * (3 + (si
 
 template <int NB, int M>
 __global__ void __launch_bounds__(MM_THREADS, 2)
-mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, float k2, float A1, float A2,
-                float per, float lim_tail, float lim_skip, float *__restrict__ partial) {
+mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, float uu, float k2, float A1, float A2,
+                float spread_max, float per, float lim_tail, float lim_skip, float *__restrict__ partial) {
     static_assert(NB % 4 == 0 && NB <= 16 && M >= 0 && M <= 4, "trajectories per group, form");
     constexpr int GS = mm_stride(NB), NT = MM_TJ / kTileCols;
     constexpr bool CW = M >= 2, HAS_TAIL = M != 1;
@@ -42,7 +49,7 @@ mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, floa
     const int64_t j0 = (int64_t)blockIdx.y * jchunk, j1 = min(n_pad, j0 + jchunk);
     const float iper = per > 0.f ? 1.f / per : 0.f;
     const float4 c = __ldg(nd.pc + row0 / kPassRows), e = __ldg(nd.pe + row0 / kPassRows);
-    const bool local = c.w == 1.f && !(per > 0.f);  // else differences, periodic ones reduced per pair
+    const bool local = c.w == 1.f && e.w <= spread_max && !(per > 0.f);  // else differences, periodic ones per pair
     u64 xi[MM_R], yi[MM_R], zi[MM_R], h1[MM_R], h2[MM_R];
 #pragma unroll
     for (int r = 0; r < MM_R; ++r) {
@@ -60,7 +67,7 @@ mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, floa
         h1[r] = f2_dup(w.x);
         h2[r] = f2_dup(w.y);
     }
-    const u64 nk2 = f2_dup(-k2), cxp = f2_dup(c.x), cyp = f2_dup(c.y), czp = f2_dup(c.z);
+    const u64 uup = f2_dup(uu), nk2 = f2_dup(-k2), cxp = f2_dup(c.x), cyp = f2_dup(c.y), czp = f2_dup(c.z);
     const u64 ipp = f2_dup(iper), npp = f2_dup(-per), mgp = f2_dup(kRintMagic);
     u64 acc[MM_R][NB / 2];
 #pragma unroll
@@ -118,7 +125,7 @@ mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, floa
                 const int q = t0 + qq;
                 const u64 xt = f2_sub(f2_pack(xs[q], xs[q + 32]), cxp), yt = f2_sub(f2_pack(ys[q], ys[q + 32]), cyp),
                           zt = f2_sub(f2_pack(zs[q], zs[q + 32]), czp);
-                const u64 nj = f2_fma(zt, zt, f2_fma(yt, yt, f2_mul(xt, xt)));
+                const u64 nj = f2_mul(f2_fma(zt, zt, f2_fma(yt, yt, f2_mul(xt, xt))), uup);
                 u64 w[MM_R];
 #pragma unroll
                 for (int r = 0; r < MM_R; ++r)
@@ -143,7 +150,7 @@ mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, floa
                         dx = f2_wrap(dx, ipp, npp, mgp);
                         dy = f2_wrap(dy, ipp, npp, mgp);
                     }
-                    w[r] = weight(PerTag<false>{}, r, f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))));
+                    w[r] = weight(PerTag<false>{}, r, f2_mul(f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))), uup));
                 }
                 add(w, q);
             }
@@ -235,18 +242,22 @@ SplitPlan multi_plan(const nf_operator *op) { return plan_splits(op->n_pad, MM_R
 // Trajectories b0 .. B - 1 (at most 16), the width rounded up to 4, 8, 12 or 16.
 nf_status launch_multi(nf_operator *op, int B, int b0, cudaStream_t s) {
     const nf_kernel &k = op->kp;
-    const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
+    const ExactUnits &eu = op->eu;
     const SplitPlan pl = multi_plan(op);
     const int group = B - b0;
+    // rows within n_i of kMultiSpread, in units of the narrower Gaussian evaluated
+    const float spread = kMultiSpread * (op->form >= 2 ? eu.k2 : (op->form == 0 ? 1.f / std::max(1.f, eu.k2) : 1.f));
     float tail, skip;
     class_limits(op, &tail, &skip);
+    tail /= eu.uu;  // boxes are in stored units
+    skip /= eu.uu;
     const dim3 grid((unsigned)ceil_div(op->n, MM_ROWS), (unsigned)pl.splits, 1);
     auto form = [&](auto nb_tag) {
         constexpr int NB = decltype(nb_tag)::value;
         auto go = [&](auto kernel) {
-            return launch_dependent(kernel, grid, MM_THREADS, mm_smem_bytes(NB), s, !op->profile, sym_nodes(op),
-                                    (const float *)op->g, B, b0, pl.jchunk, k2, k.A1, k.A2, mf_period(op), tail,
-                                    skip, op->partial);
+            return launch_dependent(kernel, grid, MM_THREADS, mm_smem_bytes(NB), s, !op->profile, exact_nodes(op),
+                                    (const float *)op->g, B, b0, pl.jchunk, eu.uu, eu.k2, k.A1, k.A2, spread, eu.per,
+                                    tail, skip, op->partial);
         };
         switch (op->form) {
             case 1: return go(mf_multi_kernel<NB, 1>);

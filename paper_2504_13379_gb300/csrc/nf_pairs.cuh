@@ -46,6 +46,27 @@ __device__ __forceinline__ float f2_fold(u64 x) {
     f2_unpack(x, lo, hi);
     return lo + hi;
 }
+// The SFU's ex2 is low by 3e-8 on average over the exponents of a planar Gaussian (measured over 2^20
+// arguments; rms 5.5e-8), its powers e2^M by about twice that.
+constexpr float kEx2Low = 3.1e-8f;
+
+// s 2^x (1 + up) for -100 < x <= 0, rounded about once: 2^r - 1 for the fraction r of x, |r| <= 1/2, by its
+// Taylor series in r ln 2 to degree 8 (remainder below 4e-10), added to s in one FMA.  For the
+// row factors of the expanded forms: their error is common to a row's whole sum, and the
+// difference of the two Gaussians' sums magnifies it.  exp2f (two units in the last place) and the
+// products around it made up most of the 1e-7 that sums of several trajectories were off.
+__device__ __forceinline__ float scale_pow2(float s, float x, float up) {
+    const float k = rintf(x), r = x - k;
+    float p = 1.3215487e-6f;              // (ln 2)^8 / 8!
+    p = fmaf(p, r, 1.5252734e-5f);        // (ln 2)^7 / 7!
+    p = fmaf(p, r, 1.5403530e-4f);        // ...
+    p = fmaf(p, r, 1.3333558e-3f);
+    p = fmaf(p, r, 9.6181291e-3f);
+    p = fmaf(p, r, 5.5504109e-2f);
+    p = fmaf(p, r, 2.4022651e-1f);
+    p = fmaf(p, r, 6.9314718e-1f);        // ln 2
+    return fmaf(s, fmaf(p, r, up), s) * __int_as_float((127 + (int)k) << 23);
+}
 __device__ __forceinline__ u64 f2_dup(float v) { return f2_pack(v, v); }
 __device__ __forceinline__ u64 f2_lo(float4 v) { return f2_pack(v.x, v.y); }
 __device__ __forceinline__ u64 f2_hi(float4 v) { return f2_pack(v.z, v.w); }
@@ -151,6 +172,12 @@ inline SymNodes sym_nodes(const nf_operator *op) {
     return SymNodes{op->xyz, op->rg, op->rw, op->pc, op->pe, op->tc, op->te, op->n, op->n_pad};
 }
 
+// The exact set (nf_operator::xyz2): coordinates times a power of two, so differences of the caller's
+// coordinates are rounded once; the exponent of a squared distance r2 is uu r2 (ExactUnits), one
+// multiplication per column of a pass, or per pair in the difference forms.
+inline SymNodes exact_nodes(const nf_operator *op) {
+    return SymNodes{op->xyz2, op->rg2, op->rw2, op->pc2, op->pe2, op->tc2, op->te2, op->n, op->n_pad};
+}
 // Lower bound of the squared distance between the nodes of two boxes (centre c, half extents
 // h); per > 0: nearest images in x and y.  A box with a non-finite node has infinite half
 // extents, which gives 0.

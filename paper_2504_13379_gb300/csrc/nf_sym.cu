@@ -83,7 +83,23 @@ float mf_unit(const nf_operator *op) {
 // The kernel's period in the units of the stored coordinates; 0 for the Euclidean distance.
 float mf_period(const nf_operator *op) { return op->kp.period > 0.f ? op->kp.period * mf_unit(op) : 0.f; }
 
-// Squared distances (stored units) beyond which a pair of nodes takes the tail form, and beyond
+// The exact set's units.  uu and k2 are rounded once each, k2 so that the product uu k2 is the second
+// Gaussian's exponent to rounding.
+static ExactUnits exact_units(const nf_operator *op) {
+    const nf_kernel &k = op->kp;
+    const double L2E = 1.4426950408889634074, s1 = k.s1, s2 = k.s2;
+    const double e1 = L2E / (s1 * s1), e2 = L2E / (s2 * s2), e = op->form >= 2 ? e2 : e1;
+    const double p = std::min(126.0, std::max(-126.0, std::round(0.5 * std::log2(e))));
+    ExactUnits u;
+    u.unit = (float)std::exp2(p);
+    u.uu = (float)(e * std::exp2(-2.0 * p));
+    u.k2 = (float)(e2 * std::exp2(-2.0 * p) / (double)u.uu);
+    if (op->form >= 2) u.k2 = (float)((s1 * s1) / (s2 * s2));
+    u.per = k.period > 0.f ? k.period * u.unit : 0.f;
+    return u;
+}
+
+// Squared distances (exponents) beyond which a pair of nodes takes the tail form, and beyond
 // which it contributes exactly 0.
 //   skip: the wider exponential evaluated has exponent > 126 with the expanded form's row part
 //         n_i <= 4 already taken out of it; one more unit for the rounding of the box bound.
@@ -138,8 +154,9 @@ struct Box {
 };
 
 // One thread per pass of kPassRows nodes: centre of the pass, its form and box, and the row
-// operands.  Forms: 1 expanded about the centre c, r^2 = n_i + s_ij, s_ij = n_j - 2 (x_i - c).
-// (x_j - c) (rows hold -2 (x_i - c)), for rows within kSymLocalSpread of c; 0 differences (rows
+// operands.  uu: exponent per squared stored unit (1: the scaled set, else ExactUnits).  Forms: 1
+// expanded about the centre c, uu r^2 = n_i + s_ij, s_ij = n_j - 2 uu (x_i - c).(x_j - c) (rows hold
+// -2 uu (x_i - c)), for rows within spread_max of c; 0 differences (rows
 // x_i); periodic kernels: 2 differences of centred coordinates (rows x_i - c), and in forms 1
 // and 2 the columns taken at their nearest image of c.  That image is the pair's nearest image
 // unless the column lies within e (the rows' distance from c) of c's antipodal lines; such a
@@ -148,9 +165,22 @@ struct Box {
 // form 3: centred differences reduced to their nearest image pair by pair.  f1, f2 are the row
 // factors 2^(-n_i) of e1 and e2 (1 outside form 1); rw holds (c_i, -A2 f2) for width ratios
 // M >= 2, with c_i = -(A1 f1) / (A2 f2), else (A1 f1, -A2 f2).
-__global__ void sym_static_kernel(const float *__restrict__ xyz, int64_t n_pad, int M, float k2, float A1, float A2,
-                                  float per, float spread_max, float4 *__restrict__ rg, float2 *__restrict__ rw,
-                                  float4 *__restrict__ pc, float4 *__restrict__ pe) {
+struct NodeSet {  // one of the operator's two sets (blockIdx.y)
+    const float *xyz;
+    float uu, k2, per, spread_max;
+    float4 *rg;
+    float2 *rw;
+    float4 *pc, *pe, *tc, *te;
+};
+struct NodeSets {
+    NodeSet s[2];
+};
+__global__ void sym_static_kernel(const __grid_constant__ NodeSets sets, int64_t n_pad, int M, float A1, float A2) {
+    const NodeSet &ns = sets.s[blockIdx.y];
+    const float *xyz = ns.xyz;
+    const float uu = ns.uu, k2 = ns.k2, per = ns.per, spread_max = ns.spread_max;
+    float4 *rg = ns.rg, *pc = ns.pc, *pe = ns.pe;
+    float2 *rw = ns.rw;
     const int64_t ps = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (ps >= n_pad / kPassRows) return;
     const int64_t r0 = ps * kPassRows;
@@ -162,12 +192,14 @@ __global__ void sym_static_kernel(const float *__restrict__ xyz, int64_t n_pad, 
         const float dx = xyz[r0 + r] - c.x, dy = xyz[n_pad + r0 + r] - c.y, dz = xyz[2 * n_pad + r0 + r] - c.z;
         spread = fmaxf(spread, dx * dx + dy * dy + dz * dz);
     }
+    const float far = sqrtf(spread);  // the rows' largest distance from the centre
+    spread *= uu;                     // as an exponent
     bool local = spread <= spread_max;
     int form = local ? 1 : 0;
     if (per > 0.f) {
         const float wide = M > 0 ? 1.f : fminf(1.f, k2);  // exponent of the wider Gaussian per unit of r^2
-        const float m = 0.5f * per - sqrtf(spread);
-        if (m > 0.f && wide * m * m >= 160.f) {
+        const float m = 0.5f * per - far;
+        if (m > 0.f && wide * uu * m * m >= 160.f) {
             form = local ? 1 : 2;
         } else {
             form = 3;
@@ -182,19 +214,21 @@ __global__ void sym_static_kernel(const float *__restrict__ xyz, int64_t n_pad, 
     for (int r = 0; r < kPassRows; ++r) {
         const int64_t k = r0 + r;
         const float px = xyz[k], py = xyz[n_pad + k], pz = xyz[2 * n_pad + k];
-        const float x = local ? -2.f * (px - c.x) : (centred ? px - c.x : px);
-        const float y = local ? -2.f * (py - c.y) : (centred ? py - c.y : py);
-        const float z = local ? -2.f * (pz - c.z) : pz;  // z never wraps
-        const float ni = local ? 0.25f * (x * x + y * y + z * z) : 0.f;
-        const float f1 = exp2f(M > 0 ? -(float)M * ni : -ni), f2 = exp2f(M > 0 ? -ni : -k2 * ni);
+        const float m2 = -2.f * uu;
+        const float x = local ? m2 * (px - c.x) : (centred ? px - c.x : px);
+        const float y = local ? m2 * (py - c.y) : (centred ? py - c.y : py);
+        const float z = local ? m2 * (pz - c.z) : pz;  // z never wraps
+        const float ni = local ? 0.25f / uu * (x * x + y * y + z * z) : 0.f;
         rg[k] = make_float4(x, y, z, ni);
-        rw[k] = make_float2(M >= 2 ? -(A1 * f1) / (A2 * f2) : A1 * f1, -A2 * f2);
+        rw[k] = make_float2(M >= 2 ? scale_pow2(-(A1 / A2), -(float)(M - 1) * ni, kEx2Low) : scale_pow2(A1, -ni, kEx2Low),
+                            scale_pow2(-A2, M > 0 ? -ni : -k2 * ni, kEx2Low));
     }
 }
 
 // One warp per tile of kTileCols nodes: its box.
-__global__ void sym_tiles_kernel(const float *__restrict__ xyz, int64_t n_pad, float4 *__restrict__ tc,
-                                 float4 *__restrict__ te) {
+__global__ void sym_tiles_kernel(const __grid_constant__ NodeSets sets, int64_t n_pad) {
+    const float *xyz = sets.s[blockIdx.y].xyz;
+    float4 *tc = sets.s[blockIdx.y].tc, *te = sets.s[blockIdx.y].te;
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (t >= n_pad / kTileCols) return;
@@ -337,8 +371,8 @@ row_bitonic_local_kernel(unsigned long long *__restrict__ keys, int blk, int64_t
 // q = 0 (so that it contributes nothing).
 __global__ void pack_sorted_kernel(const float *__restrict__ x, const float *__restrict__ q,
                                    const unsigned long long *__restrict__ keys, int64_t n, int64_t n_pad, float unit,
-                                   float4 *__restrict__ x4, float *__restrict__ xyz, float *__restrict__ qp,
-                                   int *__restrict__ perm) {
+                                   float unit2, float4 *__restrict__ x4, float *__restrict__ xyz,
+                                   float *__restrict__ xyz2, float *__restrict__ qp, int *__restrict__ perm) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_pad) return;
     const int64_t j = (int64_t)(keys[min(p, n - 1)] & 0xffffffffull);
@@ -348,6 +382,9 @@ __global__ void pack_sorted_kernel(const float *__restrict__ x, const float *__r
     xyz[p] = a * unit;
     xyz[n_pad + p] = b * unit;
     xyz[2 * n_pad + p] = c * unit;
+    xyz2[p] = a * unit2;
+    xyz2[n_pad + p] = b * unit2;
+    xyz2[2 * n_pad + p] = c * unit2;
     qp[p] = p < n ? q[j] : 0.f;
 }
 
@@ -361,18 +398,25 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     // (m < 2 n_pad of 8 bytes) take rg's place until sym_static_kernel writes it.
     const int64_t np = n_pad / kPassRows, nt = n_pad / kTileCols;
     unsigned char *mem = nullptr;
-    NF_CUDA_TRY(cudaMalloc(&mem, sizeof(float4) * (2 * n_pad + 2 * np + 2 * nt) + sizeof(float2) * n_pad +
-                                     (4 * sizeof(float) + sizeof(int)) * n_pad + 64));
+    NF_CUDA_TRY(cudaMalloc(&mem, sizeof(float4) * (3 * n_pad + 4 * np + 4 * nt) + 2 * sizeof(float2) * n_pad +
+                                     (7 * sizeof(float) + sizeof(int)) * n_pad + 64));
     op->rg = reinterpret_cast<float4 *>(mem);
     op->x4 = op->rg + n_pad;
     op->pc = op->x4 + n_pad;
     op->pe = op->pc + np;
     op->tc = op->pe + np;
     op->te = op->tc + nt;
-    op->xyz = reinterpret_cast<float *>(op->te + nt);  // n_pad is a multiple of 1024: each array stays aligned
-    op->q = op->xyz + 3 * n_pad;
+    op->rg2 = op->te + nt;
+    op->pc2 = op->rg2 + n_pad;
+    op->pe2 = op->pc2 + np;
+    op->tc2 = op->pe2 + np;
+    op->te2 = op->tc2 + nt;
+    op->xyz = reinterpret_cast<float *>(op->te2 + nt);  // n_pad is a multiple of 1024: each array stays aligned
+    op->xyz2 = op->xyz + 3 * n_pad;
+    op->q = op->xyz2 + 3 * n_pad;
     op->rw = reinterpret_cast<float2 *>(op->q + n_pad);
-    op->perm = reinterpret_cast<int *>(op->rw + n_pad);
+    op->rw2 = op->rw + n_pad;
+    op->perm = reinterpret_cast<int *>(op->rw2 + n_pad);
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(op->rg);
     float *box = reinterpret_cast<float *>(op->perm + n_pad);
     row_bbox_kernel<<<1, 1024, 0, s>>>(x, n, box);
@@ -384,17 +428,18 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
             row_bitonic_kernel<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(keys, m, jj, kk);
         row_bitonic_local_kernel<<<(unsigned)(m / blk), SORT_BLK / 2, 0, s>>>(keys, blk, kk, kk);
     }
-    pack_sorted_kernel<<<(unsigned)ceil_div(n_pad, 256), 256, 0, s>>>(x, q, keys, n, n_pad, mf_unit(op), op->x4,
-                                                                     op->xyz, op->q, op->perm);
-    // the threshold of the expanded form in the stored units, for the narrower of the Gaussians that
-    // the forward sums evaluate
+    const ExactUnits eu = op->eu = exact_units(op);
+    pack_sorted_kernel<<<(unsigned)ceil_div(n_pad, 256), 256, 0, s>>>(x, q, keys, n, n_pad, mf_unit(op), eu.unit, op->x4,
+                                                                     op->xyz, op->xyz2, op->q, op->perm);
+    // the threshold of the expanded form as an exponent, for the narrower of the Gaussians that the
+    // forward sums evaluate
     const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
-    const float spread = op->form >= 2   ? kSymLocalSpread * k2
-                         : op->form == 0 ? kSymLocalSpread / std::max(1.f, k2)
-                                         : kSymLocalSpread;
-    sym_static_kernel<<<(unsigned)ceil_div(np, 128), 128, 0, s>>>(op->xyz, n_pad, op->form, k2, k.A1, k.A2,
-                                                                 mf_period(op), spread, op->rg, op->rw, op->pc, op->pe);
-    sym_tiles_kernel<<<(unsigned)ceil_div(32 * nt, 128), 128, 0, s>>>(op->xyz, n_pad, op->tc, op->te);
+    const float narrow = op->form >= 2 ? k2 : (op->form == 0 ? 1.f / std::max(1.f, k2) : 1.f);
+    const float most = kSymLocalSpread * narrow;
+    const NodeSets sets{{{op->xyz, 1.f, k2, mf_period(op), most, op->rg, op->rw, op->pc, op->pe, op->tc, op->te},
+                         {op->xyz2, eu.uu, eu.k2, eu.per, most, op->rg2, op->rw2, op->pc2, op->pe2, op->tc2, op->te2}}};
+    sym_static_kernel<<<dim3((unsigned)ceil_div(np, 128), 2), 128, 0, s>>>(sets, n_pad, op->form, k.A1, k.A2);
+    sym_tiles_kernel<<<dim3((unsigned)ceil_div(32 * nt, 128), 2), 128, 0, s>>>(sets, n_pad);
     float hbox[6] = {0, 0, 0, 0, 0, 0};
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(hbox, box, sizeof(hbox), cudaMemcpyDeviceToHost, s);
@@ -409,9 +454,15 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
 // 1 FMA row sum, 1 FMA column sum in the full class; 3 FMA, row and column FMA in the tail class.
 // D2: every node has the same z (flat domains), so the z terms of the distance vanish
 // identically and are left out (bit-identical sums, one FMA fewer per pair).
+// Blocks of 256 and 128 nodes (sets below ~13,300 nodes) work on the exact set: with coordinates
+// rounded to exponent units two and three trajectories were 1.2 to 2 times as far from FP64 as with
+// the kernel that formed their differences before (0.8e-7 -> 1.1e-7 relative L2).  The larger
+// blocks keep the scaled set, whose columns need one multiplication less (1.5 to 2 % of a sum).
+constexpr bool sym_exact(int blk) { return blk <= 256; }
+
 template <int M, int BLK, bool D2>
 __global__ void __launch_bounds__(MS_THREADS, 2)
-mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float k2, float per, float lim_tail,
+mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float uu, float k2, float per, float lim_tail,
               float lim_skip, float *__restrict__ partial, const int *__restrict__ pairs) {
     static_assert(M >= 0 && M <= 4, "form M: 0 general, 1 one Gaussian (A2 = 0), 2-4 width ratio");
     static_assert(BLK >= 128 && BLK <= 1024 && (BLK & (BLK - 1)) == 0, "block size");
@@ -424,6 +475,7 @@ mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float k2, floa
     // unordered pair instead of 9 (separate e1 and e2 row sums, two column FMAs).
     constexpr bool CW = M >= 2;
     constexpr bool HAS_TAIL = M != 1;
+    constexpr bool EXACT = sym_exact(BLK);  // nd is the exact set, uu its exponent per squared unit
     extern __shared__ __align__(16) float ms_smem[];
     float *xs = ms_smem, *ys = xs + BLK, *zs = ys + BLK, *gs = zs + BLK;
     // per row: operands and first weight (mx, my, mz, c_i; M < 2: A1 f1 g_i), factors, and the
@@ -507,7 +559,7 @@ mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float k2, floa
     cp_async_wait_all();
     __syncthreads();
 
-    const u64 nk2 = f2_dup(-k2);
+    const u64 nk2 = f2_dup(-k2), uup = f2_dup(uu);
     const u64 ipp = f2_dup(iper), npp = f2_dup(-per), mgp = f2_dup(kRintMagic);
     const float4 *xs4 = reinterpret_cast<const float4 *>(xs), *ys4 = reinterpret_cast<const float4 *>(ys);
     const float4 *zs4 = reinterpret_cast<const float4 *>(zs), *gs4 = reinterpret_cast<const float4 *>(gs);
@@ -621,6 +673,7 @@ mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float k2, floa
                 for (int h = 0; h < 2; ++h) {
                     nj[h] = f2_fma(yt[h], yt[h], f2_mul(xt[h], xt[h]));
                     if constexpr (!D2) nj[h] = f2_fma(zt[h], zt[h], nj[h]);
+                    if constexpr (EXACT) nj[h] = f2_mul(nj[h], uup);
                 }
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
@@ -668,8 +721,10 @@ mf_sym_kernel(SymNodes nd, const float *g_all, int B, int b_base, float k2, floa
                             dx = f2_wrap(dx, ipp, npp, mgp);
                             dy = f2_wrap(dy, ipp, npp, mgp);
                         }
-                        const u64 r2xy = f2_fma(dy, dy, f2_mul(dx, dx));
-                        accum(r, D2 ? r2xy : f2_fma(dz, dz, r2xy), gj[h], cacc[h]);
+                        u64 r2 = f2_fma(dy, dy, f2_mul(dx, dx));
+                        if constexpr (!D2) r2 = f2_fma(dz, dz, r2);
+                        if constexpr (EXACT) r2 = f2_mul(r2, uup);
+                        accum(r, r2, gj[h], cacc[h]);
                     }
                 }
                 add_cols(q, cacc);
@@ -739,21 +794,25 @@ nf_status sym_init_attrs() {
 template <int BLK, bool D2>
 static cudaError_t launch_sym_blk(nf_operator *op, int B, int b_base, cudaStream_t s) {
     const nf_kernel &k = op->kp;
-    const float k2 = (k.s1 * k.s1) / (k.s2 * k.s2);
+    constexpr bool EXACT = sym_exact(BLK);
+    const ExactUnits &eu = op->eu;
+    const float uu = EXACT ? eu.uu : 1.f, k2 = EXACT ? eu.k2 : (k.s1 * k.s1) / (k.s2 * k.s2);
     const int64_t nb = op->n_pad / BLK;
     // blockIdx.z: trajectory b_base + z of the B in the partial-sum layout
     dim3 grid((unsigned)(op->mf_cull ? op->cull_live : nb * (nb + 1) / 2), 1, (unsigned)(B - b_base));
     const size_t smem = ms_smem_bytes(BLK);
-    const SymNodes nd = sym_nodes(op);
+    const SymNodes nd = EXACT ? exact_nodes(op) : sym_nodes(op);
     const int *pairs = op->mf_cull ? op->cull_pairs : nullptr;
-    const float per = mf_period(op);
+    const float per = EXACT ? eu.per : mf_period(op);
     float tail, skip;
     class_limits(op, &tail, &skip);
+    tail /= uu;  // boxes are in stored units
+    skip /= uu;
     const float *g = op->g;
     float *partial = op->partial;
     auto go = [&](auto kernel) {
-        return launch_dependent(kernel, grid, MS_THREADS, smem, s, !op->profile, nd, g, B, b_base, k2, per, tail, skip,
-                                partial, pairs);
+        return launch_dependent(kernel, grid, MS_THREADS, smem, s, !op->profile, nd, g, B, b_base, uu, k2, per, tail,
+                                skip, partial, pairs);
     };
     switch (op->form) {
         case 1: return go(mf_sym_kernel<1, BLK, D2>);
