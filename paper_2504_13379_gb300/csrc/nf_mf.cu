@@ -653,6 +653,7 @@ static nf_status mf_init_attrs_device() {
     NF_TRY(multi_init_attrs());
     NF_CUDA_TRY((set_mf_attr<1, 2>()));
     NF_CUDA_TRY((set_mf_attr<1, 4>()));
+    NF_CUDA_TRY((set_mf_attr<8, 4>()));
     NF_CUDA_TRY((set_mf_attr<16, 2>()));
     NF_CUDA_TRY((set_mf_attr<16, 4>()));
     return NF_OK;
@@ -1031,6 +1032,26 @@ nf_status mf_set_cull(nf_operator *op, int enable, int64_t *live_out, int64_t *t
     return NF_OK;
 }
 
+// The same column splits for a kernel of R rows per warp.
+static SplitPlan rows_of(SplitPlan pl, int64_t n_pad, int R) {
+    pl.rows_per_block = MF_WARPS * R;
+    pl.row_blocks = n_pad / pl.rows_per_block;
+    return pl;
+}
+
+// Groups of exactly 8 take the scalar kernel, too, in the general form where few tiles are far enough to be
+// skipped (the wider Gaussian reaches over 0.7 of the nodes' bounding box's diagonal): two
+// exponentials per pair are then needed nearly everywhere, and the packed kernel's operands keep its
+// FMA pipe at half rate.  Per sum, packed / scalar, (1.2, 0.08, 0.6, 0.25) on an ellipsoid of diameter 2: n = 20,000
+// 342 / 333 us, 30,000 748 / 716, 50,000 1,997 / 1,854; (1.2, 0.13, 0.6, 0.04), which skips: 323 / 334,
+// 677 / 715, 1,742 / 1,853.
+static bool scalar_8(const nf_operator *op) {
+    if (op->form != 0 || op->n_pad < 16384 || op->kp.period > 0.f) return false;
+    float tail, skip;
+    class_limits(op, &tail, &skip);
+    return op->span2 <= 2.f * skip;
+}
+
 nf_status launch_mf_pair(nf_operator *op, int B, cudaStream_t s, int *splits_out) {
     if (B <= kSymMaxB && use_sym(op)) {  // symmetric kernel, one partial slot per node block
         NF_TRY(launch_sym(op, B, 0, s));
@@ -1051,19 +1072,31 @@ nf_status launch_mf_pair(nf_operator *op, int B, cudaStream_t s, int *splits_out
     }
     // several: groups of exactly 16 on the scalar kernel, the rest on the packed one, over the same
     // column splits
-    SplitPlan pl = multi_plan(op);
+    const SplitPlan pl = multi_plan(op);
     *splits_out = pl.splits;
-    const int full = B / 16;
+    const int full = B / 16, R = mf_rows_per_warp(op->n_pad);
     if (full > 0) {
-        const int R = mf_rows_per_warp(op->n_pad);
-        pl.rows_per_block = MF_WARPS * R;
-        pl.row_blocks = op->n_pad / pl.rows_per_block;
+        const SplitPlan sixteen = rows_of(pl, op->n_pad, R);
         if (R == 4)
-            NF_TRY((launch_mf_group<16, 4>(op, B, 0, full, pl, s)));
+            NF_TRY((launch_mf_group<16, 4>(op, B, 0, full, sixteen, s)));
         else
-            NF_TRY((launch_mf_group<16, 2>(op, B, 0, full, pl, s)));
+            NF_TRY((launch_mf_group<16, 2>(op, B, 0, full, sixteen, s)));
     }
-    return B > 16 * full ? launch_multi(op, B, 16 * full, s) : NF_OK;
+    const int left = B - 16 * full;
+    if (left == 1) {
+        // One more trajectory: the packed kernel, over the same splits, instead of a group of four.  Per sum of
+        // 17 trajectories (ratio-4 kernel), four / one: n = 8,000 166 / 163 us, 15,000 464 / 450, 30,000
+        // 1,545 / 1,429; eight rows and 1,024-column tiles measured the same.
+        if (R == 4)
+            launch_packed<4, 512>(op, B, 16 * full, 1, rows_of(pl, op->n_pad, 4), s);
+        else
+            launch_packed<2, 512>(op, B, 16 * full, 1, rows_of(pl, op->n_pad, 2), s);
+        NF_CUDA_TRY(cudaGetLastError());
+        return NF_OK;
+    }
+    if (left == 8 && scalar_8(op))
+        return launch_mf_group<8, 4>(op, B, 16 * full, 1, rows_of(pl, op->n_pad, 4), s);
+    return left > 0 ? launch_multi(op, B, 16 * full, s) : NF_OK;
 }
 
 // Launch plan of launch_mf_pair_single: at most max_splits column splits.

@@ -446,6 +446,10 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     op->planar = (e == cudaSuccess && hbox[2] == hbox[5]) ? 1 : 0;  // one z for every node
     if (e != cudaSuccess) return cuda_fail(e, "node order", __FILE__, __LINE__);
+    for (int d = 0; d < 3; ++d) {
+        const float w = (hbox[3 + d] - hbox[d]) * mf_unit(op);
+        op->span2 += w * w;
+    }
     return NF_OK;
 }
 
