@@ -424,15 +424,15 @@ nf_status adj_autotune(nf_operator *op, const float *nu, const float *g, int B, 
     if (op->adj_r) return NF_OK;
     // 512-node blocks only on the automatic schedule without culling: an explicit symmetric
     // schedule pins the block size, and the culled pass's live-pair lists use 1,024-node
-    // blocks.  The choice is cached per (device, node count, kernel form, whether 512 is
+    // blocks.  The choice is cached per (device, node count, kernel form, tune_class, whether 512 is
     // allowed), so operators on the same node set run the same shape (culled and unculled
     // gradients then agree bit for bit).
     static std::mutex mu;
-    static std::map<std::tuple<int, int64_t, int, bool>, std::pair<int, int>> cache;
+    static std::map<std::tuple<int, int64_t, int, int, bool>, std::pair<int, int>> cache;
     const bool cull = op->mf_cull && op->adj_pairs;
     const int64_t nb1024 = op->n_pad / 1024, pairs1024 = nb1024 * (nb1024 + 1) / 2;
     const bool try512 = !cull && op->mf_sched == NF_MF_AUTO && pairs1024 < 8 * (int64_t)num_sms();
-    const auto key = std::make_tuple(op->device, op->n_pad, op->form, try512);
+    const auto key = std::make_tuple(op->device, op->n_pad, op->form, op->tune_class, try512);
     {
         std::lock_guard<std::mutex> lock(mu);
         auto it = cache.find(key);

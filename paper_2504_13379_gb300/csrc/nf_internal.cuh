@@ -261,6 +261,7 @@ struct nf_operator {
     float2 *rw2 = nullptr;
     float4 *pc2 = nullptr, *pe2 = nullptr, *tc2 = nullptr, *te2 = nullptr;
     ExactUnits eu{};
+    int tune_class = 0;      // what the timed choices of launch shape depend on besides n_pad and form
     float span2 = 0.f;       // squared diagonal of the nodes' bounding box, as an exponent (like xyz)
     int mf_variant = -1;     // launch shape of the packed pair kernel
     int adj_r = 0;           // rows per warp of the adjoint pair kernel (0: not yet timed; 4 or 8)

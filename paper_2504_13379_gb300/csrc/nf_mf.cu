@@ -849,11 +849,11 @@ void mf_launch_shape(nf_operator *op, int *R, int *TJ, int *splits) {
 static int mf_rows_per_warp(int64_t n_pad) { return n_pad >= 16384 ? 4 : 2; }
 
 // Time the symmetric kernel's node blocks (1,024, or 512 where those give too few CTAs) once on
-// this operator's nodes and keep the faster (cached per device, padded size and form).  Runs
+// this operator's nodes and keep the faster (cached per device, padded size, form and tune_class).  Runs
 // outside any stream capture.
 nf_status mf_autotune(nf_operator *op, cudaStream_t s) {
     static std::mutex mu;
-    static std::map<std::tuple<int, int64_t, int>, int> cache;
+    static std::map<std::tuple<int, int64_t, int, int>, int> cache;
     op->mf_variant = default_variant(op->n_pad);
     if (!sym_layout_fits(op)) return NF_OK;  // packed by default
     if (3 * sym_pairs_1024(op) < 2 * (int64_t)num_sms()) {
@@ -863,7 +863,7 @@ nf_status mf_autotune(nf_operator *op, cudaStream_t s) {
     // 512-node blocks only where 1,024-node pairs fill fewer than four waves of two CTAs per
     // SM (n below ~49,000): four times the CTAs even out the last wave there
     if (sym_pairs_1024(op) >= 8 * (int64_t)num_sms()) return NF_OK;
-    const auto key = std::make_tuple(op->device, op->n_pad, op->form);
+    const auto key = std::make_tuple(op->device, op->n_pad, op->form, op->tune_class);
     {
         std::lock_guard<std::mutex> lock(mu);
         auto it = cache.find(key);

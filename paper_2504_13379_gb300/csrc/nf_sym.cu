@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -175,7 +176,8 @@ struct NodeSet {  // one of the operator's two sets (blockIdx.y)
 struct NodeSets {
     NodeSet s[2];
 };
-__global__ void sym_static_kernel(const __grid_constant__ NodeSets sets, int64_t n_pad, int M, float A1, float A2) {
+__global__ void sym_static_kernel(const __grid_constant__ NodeSets sets, int64_t n_pad, int M, float A1, float A2,
+                                  int *__restrict__ count) {
     const NodeSet &ns = sets.s[blockIdx.y];
     const float *xyz = ns.xyz;
     const float uu = ns.uu, k2 = ns.k2, per = ns.per, spread_max = ns.spread_max;
@@ -205,6 +207,10 @@ __global__ void sym_static_kernel(const __grid_constant__ NodeSets sets, int64_t
             form = 3;
             local = false;
         }
+    }
+    if (blockIdx.y == 0) {  // expanded passes of the scaled set
+        const unsigned act = __activemask(), loc = __ballot_sync(act, form == 1);
+        if ((int)(threadIdx.x & 31) == __ffs(act) - 1) atomicAdd(count, __popc(loc));
     }
     pc[ps] = make_float4(c.x, c.y, c.z, (float)form);
     float4 he = bx.half(c);
@@ -255,7 +261,8 @@ __global__ void sym_tiles_kernel(const __grid_constant__ NodeSets sets, int64_t 
 // its place.
 
 // Bounding box of the n nodes (one block): box = {lo x, lo y, lo z, hi x, hi y, hi z}.
-__global__ void row_bbox_kernel(const float *__restrict__ x, int64_t n, float *__restrict__ box) {
+__global__ void row_bbox_kernel(const float *__restrict__ x, int64_t n, float *__restrict__ box, int *__restrict__ count) {
+    if (threadIdx.x == 0) *count = 0;
     __shared__ float red[6][32];
     float v[6] = {3.4e38f, 3.4e38f, 3.4e38f, -3.4e38f, -3.4e38f, -3.4e38f};
     for (int64_t j = threadIdx.x; j < n; j += blockDim.x)
@@ -388,6 +395,22 @@ __global__ void pack_sorted_kernel(const float *__restrict__ x, const float *__r
     qp[p] = p < n ? q[j] : 0.f;
 }
 
+// What the best node block of the symmetric kernels depends on besides the node count and the form: how far
+// the tail and skip classes reach against the nodes' extent (in steps of two of the squared
+// distance), the share of expanded passes (in quarters), and the planar and periodic variants.  Sum
+// on 512-node blocks over sum on 1,024: from 0.41 (narrow kernel, 20,000 nodes in a periodic square)
+// to 1.5 (wide general kernel, 20,000 in a cube) at one node count and form.
+static int tune_class(const nf_operator *op, double expanded) {
+    float tail, skip;
+    class_limits(op, &tail, &skip);
+    auto reach = [&](float lim) {
+        const double r = (double)lim / std::max((double)op->span2, 1e-30);
+        return std::min(31, std::max(0, 24 + (int)std::floor(std::log2(std::max(r, 1e-30)))));
+    };
+    const int share = std::min(3, (int)(4.0 * expanded));
+    return (((share * 32 + reach(tail)) * 32 + reach(skip)) * 2 + op->planar) * 2 + (op->kp.period > 0.f ? 1 : 0);
+}
+
 nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaStream_t s) {
     const int64_t n = op->n, n_pad = op->n_pad;
     const nf_kernel &k = op->kp;
@@ -419,7 +442,8 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     op->perm = reinterpret_cast<int *>(op->rw2 + n_pad);
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(op->rg);
     float *box = reinterpret_cast<float *>(op->perm + n_pad);
-    row_bbox_kernel<<<1, 1024, 0, s>>>(x, n, box);
+    int *count = reinterpret_cast<int *>(box + 6);
+    row_bbox_kernel<<<1, 1024, 0, s>>>(x, n, box, count);
     row_key_kernel<<<(unsigned)ceil_div(m, 256), 256, 0, s>>>(x, n, m, box, keys);
     const int blk = (int)std::min<int64_t>(m, SORT_BLK);
     row_bitonic_local_kernel<<<(unsigned)(m / blk), SORT_BLK / 2, 0, s>>>(keys, blk, 2, blk);
@@ -438,9 +462,9 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
     const float most = kSymLocalSpread * narrow;
     const NodeSets sets{{{op->xyz, 1.f, k2, mf_period(op), most, op->rg, op->rw, op->pc, op->pe, op->tc, op->te},
                          {op->xyz2, eu.uu, eu.k2, eu.per, most, op->rg2, op->rw2, op->pc2, op->pe2, op->tc2, op->te2}}};
-    sym_static_kernel<<<dim3((unsigned)ceil_div(np, 128), 2), 128, 0, s>>>(sets, n_pad, op->form, k.A1, k.A2);
+    sym_static_kernel<<<dim3((unsigned)ceil_div(np, 128), 2), 128, 0, s>>>(sets, n_pad, op->form, k.A1, k.A2, count);
     sym_tiles_kernel<<<dim3((unsigned)ceil_div(32 * nt, 128), 2), 128, 0, s>>>(sets, n_pad);
-    float hbox[6] = {0, 0, 0, 0, 0, 0};
+    float hbox[7] = {0, 0, 0, 0, 0, 0, 0};  // with the count behind the box
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(hbox, box, sizeof(hbox), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -450,6 +474,9 @@ nf_status mf_build_nodes(nf_operator *op, const float *x, const float *q, cudaSt
         const float w = (hbox[3 + d] - hbox[d]) * mf_unit(op);
         op->span2 += w * w;
     }
+    int expanded = 0;
+    std::memcpy(&expanded, &hbox[6], sizeof(int));
+    op->tune_class = tune_class(op, (double)expanded / (double)np);
     return NF_OK;
 }
 
