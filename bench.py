@@ -149,16 +149,25 @@ def peaks():
 # sum), plus per column and 8-row pass 3 SUB + 3 FMA (centred column and n_j) and 1 ADD
 # (column sums into shared memory): 8.875 per unordered pair in the full class; the tail class,
 # whose narrow Gaussian cannot change the FP32 sum, leaves 3 of them out (5.875); pairs whose
-# exponentials are exactly 0 in FP32 are skipped.  On the n = 100,000 torus 12 % of the tile
-# visits are full, 73 % tail and 15 % skipped: 5.35 per unordered pair.  Pair evaluations
-# count all n^2 ordered pairs of the sum.  Diagonal block pairs evaluate their ordered pairs
-# one by one, a 1/nb share of the work.  The rates these counts are divided by (FP32 FMA-pipe
-# lane operations and SFU ex2 per clock per SM) are measured in the same run by nf_probe_pipe;
-# the nominal figures (128 FP32 lanes, 16 SFU operations per clock per SM) are kept only as a
-# fallback.
+# exponentials are exactly 0 in FP32 are skipped.  The shares of the tile visits are known for
+# the n = 100,000 torus with the workload's kernel only: 12 % full, 73 % tail, 15 % skipped, 5.35
+# operations per unordered pair.  Other sizes count every pair in full, which the fraction may
+# pass where many tiles are not.  Pair evaluations count all n^2 ordered pairs of the sum.  Diagonal
+# block pairs evaluate their ordered pairs one by one, a 1/nb share of the work.  The rates these
+# counts are divided by (FP32 FMA-pipe lane operations and SFU ex2 per clock per SM) are
+# measured in the same run by nf_probe_pipe; the nominal figures (128 FP32 lanes, 16 SFU
+# operations per clock per SM) are kept only as a fallback.
 FMA_LANES_PER_CLK_SM_NOMINAL = 128.0
-LANE_OPS_PER_PAIR = (0.12 * 8.875 + 0.73 * 5.875) / 2.0
-EX2_PER_PAIR = 0.85 * 0.5
+
+
+def pair_operations(n):
+    """FMA-pipe lane operations and exponentials per ordered pair off the diagonal blocks, and what
+    they count, for the precision torus with n nodes."""
+    if n == 100000:
+        return ((0.12 * 8.875 + 0.73 * 5.875) / 2.0, 0.85 * 0.5,
+                "12 % of the tile visits in full, 73 % with one Gaussian, 15 % exactly zero")
+    return 8.875 / 2.0, 0.5, "every pair in full: the shares of the shorter tiles are not known at this size"
+
 
 # DRAM bytes (read + write) per launch from ncu captures of the current kernels:
 # the symmetric kernel on the n = 100,000 torus (--set full); tc_grouped_kernel<4> (an RK4
@@ -925,23 +934,24 @@ def run_ours(args, rank, world, local_rank):
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         mhz = clocks["sm_mhz"] or pk.get("clocks_under_load", {}).get("sm_mhz_median") or 1432.0
         nb = -(-n // 1024)
-        ops = LANE_OPS_PER_PAIR * (1.0 + 1.0 / nb)
+        ops, ex2_per_pair, counted = pair_operations(n)
+        ops *= 1.0 + 1.0 / nb
         lanes = pipes["fma_f32x2"]["per_clk_per_sm"]
         ex2 = pipes["ex2"]["per_clk_per_sm"]
         fma_peak = sms * lanes * mhz * 1e6 / ops / 1e9                      # Gpair/s on the FP32 FMA pipe
         lanes_gen = pipes["fma_f32x2_outer"]["per_clk_per_sm"]  # packed FMAs with varied operands
         fma_peak_gen = sms * lanes_gen * mhz * 1e6 / ops / 1e9
-        sfu_peak = sms * ex2 * mhz * 1e6 / (EX2_PER_PAIR * (1.0 + 1.0 / nb)) / 1e9  # Gpair/s on the SFU
+        sfu_peak = sms * ex2 * mhz * 1e6 / (ex2_per_pair * (1.0 + 1.0 / nb)) / 1e9  # Gpair/s on the SFU
         peak = min(fma_peak, sfu_peak)
         achieved = n * n / (kms * 1e-3) / 1e9
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Gpair/s", "frac": achieved / peak,
                 "traffic": MF_TRAFFIC_BYTES if n == 100000 else None, "traffic_unit": "bytes per launch",
                 "peak_basis": f"measured: {sms} SMs x {lanes:.1f} FP32 FMA-pipe lane operations/clk/SM (f32x2 "
                               f"probe in this run) x {mhz:.0f} MHz (median SM clock in the timed region) / "
-                              f"{ops:.3f} lane operations per ordered pair (symmetric kernel, expanded form, m = 4; 12 % "
-                              f"of the tile visits in full, 73 % with one Gaussian, 15 % exactly zero); "
+                              f"{ops:.3f} lane operations per ordered pair (symmetric kernel, expanded form, m = 4; "
+                              f"{counted}); "
                               f"SFU ceiling {sfu_peak:.0f} Gpair/s from {ex2:.1f} ex2/clk/SM measured and "
-                              f"{EX2_PER_PAIR:.3f} exponentials per ordered pair",
+                              f"{ex2_per_pair:.3f} exponentials per ordered pair",
                 "fma_pipe_peak": fma_peak, "sfu_peak": sfu_peak,
                 "fma_pipe_peak_varied_operands": fma_peak_gen, "frac_vs_varied_operands": achieved / fma_peak_gen,
                 "nominal_peak_128_lanes": sms * FMA_LANES_PER_CLK_SM_NOMINAL * mhz * 1e6 / ops / 1e9}
