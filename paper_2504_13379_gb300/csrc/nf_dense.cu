@@ -515,18 +515,6 @@ struct GemmSmem {
     unsigned long long b[2][GB_BK][GB_BN + 2];      // (f, f) pairs, k-major
 };
 
-typedef unsigned long long u64d;
-__device__ __forceinline__ u64d d_fma2(u64d a, u64d b, u64d c) {
-    u64d d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ u64d d_pack(float lo, float hi) {
-    u64d d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-
 template <int GB_BN>
 __global__ void __launch_bounds__(GB_THREADS, 2)
 gemm_fp32_kernel(const float *__restrict__ W, const float *__restrict__ F, int64_t n_pad, int B, int64_t kchunk,
@@ -568,13 +556,13 @@ gemm_fp32_kernel(const float *__restrict__ W, const float *__restrict__ F, int64
 #pragma unroll
         for (int p = 0; p < BLD; ++p) {
             const int idx = tid + GB_THREADS * p, c = idx >> 2, kq = idx & 3;
-            sm.b[buf][4 * kq + 0][c] = d_pack(rb[p].x, rb[p].x);
-            sm.b[buf][4 * kq + 1][c] = d_pack(rb[p].y, rb[p].y);
-            sm.b[buf][4 * kq + 2][c] = d_pack(rb[p].z, rb[p].z);
-            sm.b[buf][4 * kq + 3][c] = d_pack(rb[p].w, rb[p].w);
+            sm.b[buf][4 * kq + 0][c] = f2_dup(rb[p].x);
+            sm.b[buf][4 * kq + 1][c] = f2_dup(rb[p].y);
+            sm.b[buf][4 * kq + 2][c] = f2_dup(rb[p].z);
+            sm.b[buf][4 * kq + 3][c] = f2_dup(rb[p].w);
         }
     };
-    u64d acc[4][NC];
+    u64 acc[4][NC];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -589,7 +577,7 @@ gemm_fp32_kernel(const float *__restrict__ W, const float *__restrict__ F, int64
         if (kt + 1 < nkt) load(kt + 1);  // global loads in flight during the compute below
 #pragma unroll 4
         for (int k = 0; k < GB_BK; ++k) {
-            u64d bd[NC];
+            u64 bd[NC];
 #pragma unroll
             for (int c2 = 0; c2 < NC; c2 += 2) {
                 const int col = (c2 < 4 ? tn * 4 : 64 + tn * 4) + (c2 & 3);
@@ -599,9 +587,9 @@ gemm_fp32_kernel(const float *__restrict__ W, const float *__restrict__ F, int64
             }
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                const u64d a = *reinterpret_cast<const u64d *>(&sm.a[buf][k][2 * tm + 32 * r]);
+                const u64 a = *reinterpret_cast<const u64 *>(&sm.a[buf][k][2 * tm + 32 * r]);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) acc[r][c] = d_fma2(a, bd[c], acc[r][c]);
+                for (int c = 0; c < NC; ++c) acc[r][c] = f2_fma(a, bd[c], acc[r][c]);
             }
         }
         if (kt + 1 < nkt) store(buf ^ 1);
@@ -614,7 +602,7 @@ gemm_fp32_kernel(const float *__restrict__ W, const float *__restrict__ F, int64
         if (b >= B) continue;
 #pragma unroll
         for (int r = 0; r < 4; ++r)
-            *reinterpret_cast<u64d *>(out + (int64_t)b * n_pad + m0 + 2 * tm + 32 * r) = acc[r][c];
+            *reinterpret_cast<u64 *>(out + (int64_t)b * n_pad + m0 + 2 * tm + 32 * r) = acc[r][c];
     }
 }
 
