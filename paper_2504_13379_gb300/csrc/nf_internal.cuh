@@ -191,6 +191,14 @@ __device__ __forceinline__ long long ld_l2(const long long *p) {
     return v;
 }
 
+// Ordinary load that stays behind pdl_wait() (volatile asm keeps its order) and leaves the compiler as free
+// with the stores around it as __ldg does.
+__device__ __forceinline__ float ld_written(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, bool overlap,
                              A... args) {

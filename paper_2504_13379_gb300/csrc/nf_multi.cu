@@ -10,8 +10,8 @@
 //
 // Bound: the FP32 FMA pipe, NB + 3 to 8 lane operations per ordered pair (NB + 10 with two
 // exponentials per pair in the scalar kernel that served every width before, in groups of 16, 8,
-// 4, 2, 1).  Per sum before / now, n = 15,000: 4 trajectories 159 / 122 us, 6 285 / 172, 8 210 /
-// 174, 12 365 / 265; groups of exactly 16 stay on the scalar kernel.  Scalar accumulators in
+// 4, 2, 1).  Per sum before / now, n = 15,000: 4 trajectories 159 / 119 us, 6 285 / 170, 8 210 /
+// 172, 12 365 / 248; groups of exactly 16 stay on the scalar kernel.  Scalar accumulators in
 // place of the pairs measured the same.
 #include "nf_pairs.cuh"
 
@@ -167,12 +167,15 @@ mf_multi_kernel(SymNodes nd, const float *g, int B, int b0, int64_t jchunk, floa
             const int k = tid + t * MM_THREADS;
             const int64_t j = jt + k;
             const bool in = j < j1;
+            // The rates' loads first, and as ld_written: with plain loads, or the coordinates first, the sweeps
+            // below came out slower (n = 15,000: 8 trajectories 186 us, plain loads first 184, ld_written
+            // second 176, both 172; 12 trajectories 254, 248, 254, 248).
+            float v[NB];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) v[b] = in && b < nv ? ld_written(g + (int64_t)(b0 + b) * n_pad + j) : 0.f;
             xs[k] = in ? __ldg(nd.xyz + j) : 0.f;
             ys[k] = in ? __ldg(nd.xyz + n_pad + j) : 0.f;
             zs[k] = in ? __ldg(nd.xyz + 2 * n_pad + j) : 0.f;
-            float v[NB];
-#pragma unroll
-            for (int b = 0; b < NB; ++b) v[b] = in && b < nv ? g[(int64_t)(b0 + b) * n_pad + j] : 0.f;
 #pragma unroll
             for (int b = 0; b < NB; ++b) bad |= !(0.f * v[b] == 0.f);  // non-finite
 #pragma unroll
