@@ -250,7 +250,7 @@ __device__ __forceinline__ uint4 ld_stream_u4(const void *p) {
 // trajectory).  A warp takes 4 rows; every W value it loads meets NB vector values from L1.  HL:
 // bf16 hi + lo planes in the blocked layout, lane l on columns tile + 8 l + 256 u; else the FP32
 // plane, columns tile + 4 l + 128 u.  Bound: HBM, 4 bytes per entry whatever NB: per RK4 stage at
-// n = 30,000 on the bf16 planes 1, 2, 3, 4, 8 trajectories in 525, 529, 526, 552, 644 us (559,
+// n = 30,000 on the bf16 planes 1, 2, 3, 4, 8 trajectories in 525, 529, 526, 552, 638 us (559,
 // 1,112, 1,667, 2,219, 4,450 with one stream each).  Two CTAs per SM at 128 registers beat one
 // with more (3 trajectories 526 against 689 us).
 template <int NB, bool HL>
@@ -299,7 +299,10 @@ gemv_kernel(const void *__restrict__ W0, const uint16_t *__restrict__ Wlo, const
                 for (int v = 0; v < NB; ++v)
 #pragma unroll
                     for (int c = 0; c < C; c += 4) {
-                        const float4 f = *reinterpret_cast<const float4 *>(fp + (int64_t)v * n_pad + c);
+                        // (plain loads spill 232 bytes a thread on the bf16 planes with 8 trajectories: n = 30,000
+                        // 919 us against 638; on the FP32 plane they are the better ones: 643 against 667)
+                        const float *src = fp + (int64_t)v * n_pad + c;
+                        const float4 f = HL ? ld_written4(src) : *reinterpret_cast<const float4 *>(src);
                         fv[v][c] = f.x, fv[v][c + 1] = f.y, fv[v][c + 2] = f.z, fv[v][c + 3] = f.w;
                     }
 #pragma unroll
