@@ -115,7 +115,7 @@ nf_status ensure_workspace(nf_operator *op, int B, int splits, cudaStream_t s, b
 }
 
 SplitPlan mf_plan(nf_operator *op);
-SplitPlan dense_plan(nf_operator *op);
+SplitPlan dense_plan(nf_operator *op, int B);
 
 int nonlocal_splits(nf_operator *op, int B) {
     return (op->path == NF_MATRIX_FREE) ? mf_splits(op, B) : dense_splits(op, B);

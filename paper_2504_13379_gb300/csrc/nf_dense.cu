@@ -250,11 +250,12 @@ __device__ __forceinline__ uint4 ld_stream_u4(const void *p) {
 // trajectory).  A warp takes 4 rows; every W value it loads meets NB vector values from L1.  HL:
 // bf16 hi + lo planes in the blocked layout, lane l on columns tile + 8 l + 256 u; else the FP32
 // plane, columns tile + 4 l + 128 u.  Bound: HBM, 4 bytes per entry whatever NB: per RK4 stage at
-// n = 30,000 on the bf16 planes 1, 2, 3, 4, 8 trajectories in 525, 529, 526, 552, 638 us (559,
+// n = 30,000 on the bf16 planes 1, 2, 3, 4, 8 trajectories in 506, 529, 526, 552, 638 us (559,
 // 1,112, 1,667, 2,219, 4,450 with one stream each).  Two CTAs per SM at 128 registers beat one
-// with more (3 trajectories 526 against 689 us).
+// with more (3 trajectories 526 against 689 us); one trajectory on the bf16 planes takes three (four, at 64
+// registers, spill: 588 us).
 template <int NB, bool HL>
-__global__ void __launch_bounds__(DG_THREADS, NB == 1 && HL ? 4 : 2)
+__global__ void __launch_bounds__(DG_THREADS, NB == 1 && HL ? 3 : 2)
 gemv_kernel(const void *__restrict__ W0, const uint16_t *__restrict__ Wlo, const float *F, int64_t n_pad,
             int B, int b0, int64_t jchunk, float *__restrict__ partial) {
     constexpr int C = HL ? 8 : 4;                 // columns per load
@@ -666,10 +667,14 @@ nf_status dense_init_attrs() {
     return NF_OK;
 }
 
-SplitPlan dense_plan(nf_operator *op) {
+// The columns' splits fill whole waves of resident CTAs: two per SM for several trajectories (counted as four on
+// the bf16 planes: an even number of waves), the kernel's own number for one.
+SplitPlan dense_plan(nf_operator *op, int B) {
     int res = 0;
     if (op->path == NF_DENSE_FP32)
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, gemv_kernel<1, false>, DG_THREADS, 0);
+    else if (B > 1)
+        res = 4;
     else
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, gemv_kernel<1, true>, DG_THREADS, 0);
     return plan_splits(op->n_pad, DG_ROWS, DG_TILE, std::max(res, 1));
@@ -678,7 +683,7 @@ SplitPlan dense_plan(nf_operator *op) {
 int dense_splits(nf_operator *op, int B) {
     if (use_gemm(op, B)) return gemm_plan(op, B).splits;
     const bool sym = op->path == NF_DENSE_SYM_FP32 || op->path == NF_DENSE_SYM_BF16X2;
-    return sym ? (int)(op->n_pad / SB) : dense_plan(op).splits;
+    return sym ? (int)(op->n_pad / SB) : dense_plan(op, B).splits;
 }
 
 size_t dense_sym_entries(int64_t n_pad) {
@@ -791,7 +796,7 @@ nf_status launch_dense_gemv(nf_operator *op, int B, cudaStream_t s, int *splits_
         *splits_out = gp.splits;
         return NF_OK;
     }
-    const SplitPlan pl = dense_plan(op);
+    const SplitPlan pl = dense_plan(op, B);
     if (op->path == NF_DENSE_FP32)
         NF_TRY(launch_gemvs<false>(op, B, pl, s));
     else
