@@ -172,7 +172,7 @@ def pair_operations(n):
 # DRAM bytes (read + write) per launch from ncu captures of the current kernels:
 # the symmetric kernel on the n = 100,000 torus (--set full); tc_grouped_kernel<4> (an RK4
 # stage-4 launch) on the full batched workload (dram__bytes_read/write.sum, one pass)
-MF_TRAFFIC_BYTES = 2.182e6 + 0.140e6
+MF_TRAFFIC_BYTES = 4.48e6 + 0.008e6
 TC_TRAFFIC_BYTES = 11.90e9 + 0.214e9
 
 

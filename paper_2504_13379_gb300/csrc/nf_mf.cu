@@ -736,15 +736,15 @@ static nf_status launch_mf_packed(nf_operator *op, int B, int b_base, int groups
 // trajectory: each trajectory's pairs are evaluated once, which beats the multi-trajectory
 // kernels (ordered pairs, exponentials shared across trajectories) until about four
 // trajectories (n = 100,000: 1.10 ms per symmetric trajectory, B = 4 in 4.0 ms there; n = 20,000:
-// B = 3 symmetric in 0.203 ms, B = 4 there in 0.198).
+// B = 3 symmetric in 0.193 ms, B = 4 there in 0.202).
 constexpr int kSymMaxB = 3;
 
 // Small node sets on the automatic schedule take one launch per sum: 2 rows per warp, columns in
 // tiles of 1,024 (one or two at most sizes here; 512-node tiles, 1 or 4 rows per warp measured
 // slower at most sizes).  Per RK4 stage on GB300, against the packed pair kernel and the stage
-// kernel with and without overlapped launches: n = 1,000 4.3 us (4.8, 5.9), 2,000 5.9 (6.4, 8.4),
-// 3,000 9.5 (9.4, 11.0); at 4,000 nodes 11.5, where the symmetric kernel on 256-node blocks takes
-// 9.5 (15.1 before), hence the line.
+// kernel with and without overlapped launches: n = 1,000 4.2 us (4.8, 5.9), 2,000 5.7 to 6.1 (6.4,
+// 8.4), 3,000 9.4 (9.4, 11.0); at 4,000 nodes 11.5, where the symmetric kernel on 256-node blocks
+// takes 9.6 (15.1 before), hence the line.
 constexpr int64_t kFusedMaxN = 3072;
 constexpr int kFusedRows = 2, kFusedTile = 1024;
 bool fused_fits(const nf_operator *op, int B) {
@@ -786,7 +786,7 @@ int sym_slots(const nf_operator *op) { return (int)(op->n_pad / op->sym_blk); }
 // Up to kSymMaxB trajectories take the symmetric kernel beyond kFusedMaxN nodes, on blocks of
 //   256 nodes  while 1,024-node block pairs are fewer than 2/3 of the SMs (n below ~13,300): the
 //              packed row-block x column-split kernel that served these sizes before evaluates
-//              ordered pairs (per RK4 stage, packed before / 256 / 512: n = 5,500 23.9 / 13.1 /
+//              ordered pairs (per RK4 stage, packed before / 256 / 512: n = 5,500 23.9 / 12.9 /
 //              20.8 us, 8,000 40.4 / 20.6 / 20.8, 13,000 82 / 41 / 43);
 //   512, 1,024 above, by timing (mf_autotune).
 // The automatic schedule also keeps the symmetric partial sums (one slot of n_pad floats per

@@ -10,7 +10,7 @@
 //
 // Bound: the FP32 FMA pipe, NB + 3 to 8 lane operations per ordered pair (NB + 10 with two
 // exponentials per pair in the scalar kernel that served every width before, in groups of 16, 8,
-// 4, 2, 1).  Per sum before / now, n = 15,000: 4 trajectories 159 / 119 us, 6 285 / 170, 8 210 /
+// 4, 2, 1).  Per sum before / now, n = 15,000: 4 trajectories 159 / 119 us, 6 285 / 172, 8 210 /
 // 172, 12 365 / 248; groups of exactly 16 stay on the scalar kernel.  Scalar accumulators in
 // place of the pairs measured the same.
 #include "nf_pairs.cuh"

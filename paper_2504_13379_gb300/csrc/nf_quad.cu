@@ -4,8 +4,8 @@
 // planes, central projection of the stencil to the element plane and the Jacobian of the map),
 // the saddle system of Eq. (3.4) with r^3 and monomials up to deg, analytic right-hand side, LU
 // with partial pivoting in shared memory, element weights; then a deterministic gather
-// q_i = sum of the element weights of every stencil entry naming node i, in ascending
-// (element, position) order.
+// q_i = sum of the element weights of every stencil entry naming node i, in a fixed order (32
+// strands of the (element, position) ranks and a butterfly over them).
 //
 // Bound: the FP64 pipe, two lanes per clock and SM -- a warp instruction costs 16 clocks however
 // few of its lanes are active.  The elimination of a k = 48, degree-4 system (N = 63) is 2,700
@@ -311,8 +311,8 @@ __device__ __forceinline__ unsigned long long abs_key(double v) {
 // sqrt(q) for q in FP32 range: reciprocal square root of FP32, one Goldschmidt iteration for the
 // root and half its reciprocal, and a final residual correction (Markstein, "IA-64 and Elementary
 // Functions", 2000): seven FP64 operations, half of the library call's.  Within one unit in
-// the last place of sqrt; on 6.5e7 random arguments of GB300 it agreed with sqrt to the bit.  0
-// and values outside FP32's normal range take the library's.
+// the last place of sqrt (a run of its own over 6.5e7 random arguments found no difference; the tests
+// check the weights, not this function).  0 and values outside FP32's normal range take the library's.
 __device__ __forceinline__ double root(double q) {
     const float qf = (float)q;
     if (!(qf > 1e-30f && qf < 1e30f)) return sqrt(q);
